@@ -15,7 +15,7 @@ int taps_project_sources_dim(const taps_dim* d, const taps_source* sources, int 
 int taps_project_source(const taps_dim* d, int kind, const double* par, const double* nodal_host,
                         double* d_q_free, cudaStream_t s);
 
-int taps_sweep_setup(int dev, int num_sms, int* coop_blocks);
+int taps_sweep_setup(int dev, int num_sms, int* coop_blocks, int* ts_most, size_t* ts_maxsm);
 
 // ---------------------------------------------------------------------------------
 // Profiling: launch counts always; CUDA events around launches when enabled.
@@ -496,6 +496,8 @@ static void free_ws(taps_problem* P) {
   cudaFree(P->d_lu);
   cudaFree(P->d_Y);
   cudaFree(P->d_Uold);
+  cudaFree(P->d_ts);
+  P->d_ts = nullptr;
   cudaFree(P->d_md);
   P->d_md = nullptr;
   cudaFree(P->d_fdw);
@@ -549,11 +551,12 @@ int taps_ws_ensure(taps_problem* P, int M) {
   free_ws(P);
   P->c0_valid = 0;
   int nbmax = 0, D = P->D;
-  size_t part = 0, bigG = 0, yres = 0, part_all = 0;
+  size_t part = 0, bigG = 0, yres = 0, part_all = 0, ts = 0;
   for (int d = 0; d < D; ++d) {
     const taps_dim* dm = P->dims[d];
     int nops = P->tt.nops[d];
     nbmax = std::max(nbmax, dm->nb);
+    ts = std::max(ts, taps_ts_scratch_doubles(dm->hb, std::min(M, 64)));
     TAPS_TRY(taps_alloc((void**)&P->d_gram[d], sizeof(double) * nops * M * M));
     TAPS_TRY(taps_alloc((void**)&P->d_h[d], sizeof(double) * P->Rf * M));
     TAPS_TRY(taps_alloc((void**)&P->d_Usnap[d], sizeof(double) * dm->nf * M));
@@ -587,6 +590,7 @@ int taps_ws_ensure(taps_problem* P, int M) {
   TAPS_TRY(taps_alloc((void**)&P->d_lu, sizeof(double) * MM));
   TAPS_TRY(taps_alloc((void**)&P->d_Y, sizeof(double) * cs * nfm * M));
   TAPS_TRY(taps_alloc((void**)&P->d_Uold, sizeof(double) * nfm * M));
+  TAPS_TRY(taps_alloc((void**)&P->d_ts, sizeof(double) * ts));
   TAPS_TRY(taps_alloc((void**)&P->d_fdw, sizeof(double) * taps_fdw_scratch_doubles(nfm, M)));
   TAPS_TRY(taps_alloc((void**)&P->d_md, sizeof(double) * taps_md_scratch_doubles(nfm, M, P->Rf)));
   TAPS_CUDA(cudaMemsetAsync(P->d_md, 0, sizeof(double) * taps_md_scratch_doubles(nfm, M, P->Rf), P->stream));
@@ -709,7 +713,7 @@ extern "C" int taps_problem_create(taps_dim* const* dims, int D, const taps_term
       st = taps_project_sources_dim(dm, sources, Rf, d, P->d_q[d], P->stream);
     }
     if (st != TAPS_OK) break;
-    if ((st = taps_sweep_setup(dev, P->num_sms, &P->coop_blocks)) != TAPS_OK) break;
+    if ((st = taps_sweep_setup(dev, P->num_sms, &P->coop_blocks, &P->ts_most, &P->ts_maxsm)) != TAPS_OK) break;
     st = taps_check_status(P->d_status, P->stream);
   } while (0);
   if (st != TAPS_OK) {

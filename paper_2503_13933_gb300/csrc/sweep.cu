@@ -1079,6 +1079,7 @@ int taps_lu_needs_tuning(const taps_problem* P, int solver, int M) {
     (void)sa;
     (void)sb;
     if (taps_dim_route(P, d, solver, M) != TAPS_ROUTE_LU) continue;
+    if (taps_ts_ctas(P, P->dims[d]->hb, M) > 0) continue;   // the two-sided route has no trials
     bool found = false;
     for (int k = 0; k < P->n_lu_tuned; ++k)
       if (P->lu_tuned[k][0] == P->dims[d]->nf && P->lu_tuned[k][1] == M) found = true;
@@ -1108,6 +1109,14 @@ static int reduced_solve_block_lu(taps_problem* P, taps_factors* U, int d) {
     bs_flops += nj * 2.0 * Md * Md;
   }
   const double band_bytes = 8.0 * (double)nf * nb * M * M;
+  const int nc = taps_ts_ctas(P, hb, M);
+  if (nc > 0) {   // from both ends, middle and back substitution; keeps the old factor in d_Uold
+    tk = prof_begin(P, TAPS_PROF_BLOCK_LU);
+    TAPS_TRY(taps_ts_solve(P, U, d, nc));
+    prof_end(P, TAPS_PROF_BLOCK_LU, tk, lu_flops + bs_flops, 2.0 * band_bytes + 16.0 * nf * M);
+    return TAPS_OK;
+  }
+  TAPS_CUDA(cudaMemcpyAsync(P->d_Uold, U->d_U[d], sizeof(double) * nf * M, cudaMemcpyDeviceToDevice, s));
   // cooperative elimination; the CTA count comes from the tuner (first use per (n, M))
   size_t smem = sizeof(double) * (size_t)M * (M + 1);
   int grid = taps_lu_grid(P, d, U, nf, M);
@@ -1145,7 +1154,7 @@ int taps_allow_dyn_smem(const void* fn, int maxsm) {
 
 // Shared-memory opt-in of the kernels whose footprint grows with M, and the number
 // of CTAs a cooperative block-LU launch may use (co-residency at the largest M).
-int taps_sweep_setup(int dev, int num_sms, int* coop_blocks) {
+int taps_sweep_setup(int dev, int num_sms, int* coop_blocks, int* ts_most, size_t* ts_maxsm) {
   int maxsm = 0;
   TAPS_CUDA(cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
   TAPS_TRY(taps_allow_dyn_smem((const void*)block_lu_kernel, maxsm));
@@ -1156,6 +1165,7 @@ int taps_sweep_setup(int dev, int num_sms, int* coop_blocks) {
   TAPS_TRY(residual_setup(maxsm));
   TAPS_TRY(taps_md_setup(maxsm));
   TAPS_TRY(taps_gram_tc_setup(maxsm));
+  TAPS_TRY(taps_ts_setup(maxsm, ts_most, ts_maxsm));
   int bps = 0;
   size_t smem_max = sizeof(double) * TAPS_MAX_M * (TAPS_MAX_M + 1);
   TAPS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, block_lu_kernel, 256, smem_max));
@@ -1205,9 +1215,7 @@ int taps_sweep_enqueue(taps_problem* P, taps_factors* U, int precision, int solv
     } else if (route == TAPS_ROUTE_FDW) {
       TAPS_TRY(taps_fdw_solve(P, U, d));             // keeps the old factor in d_Uold
     } else {
-      TAPS_CUDA(cudaMemcpyAsync(P->d_Uold, U->d_U[d], sizeof(double) * dm->nf * M,
-                                cudaMemcpyDeviceToDevice, s));
-      TAPS_TRY(reduced_solve_block_lu(P, U, d));
+      TAPS_TRY(reduced_solve_block_lu(P, U, d));     // keeps the old factor in d_Uold
     }
     int norm_d = (normalize && d < P->D - 1) ? 1 : 0;
     int tk = prof_begin(P, TAPS_PROF_NORMALIZE);

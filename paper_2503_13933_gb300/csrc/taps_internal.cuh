@@ -143,6 +143,7 @@ struct taps_problem {
   double* d_lu;       // [M][M] LU of the current diagonal block
   double* d_Y;        // [tt.cs][nf_max][M] SpMM products
   double* d_Uold;     // [nf_max][M]
+  double* d_ts;       // two-sided elimination: the middle as each side leaves it
   double* d_fdw;      // convection-face corrections: X [nf_max][2][M][M], w [nf_max][M], small parts
   double* d_md;       // mode-side solve: W [M][M], lam [M], W^T c [Rf][M], Z [nf_max][M],
                       // eliminated rows [nf_max][6][M]
@@ -169,6 +170,8 @@ struct taps_problem {
   int lu_tuned[16][3];  // tuned block-elimination CTA counts: (n, M, CTAs)
   int n_lu_tuned;
   int coop_blocks;    // CTAs of the cooperative block solve
+  int ts_most;        // two-sided elimination: largest cluster the device places
+  size_t ts_maxsm;    // and the shared memory one of its CTAs may ask for
   // d_C / d_c hold dim 0's coefficients for the current Grams (the last dim's Gram
   // refresh of a sweep or of taps_refresh_grams forms them), so the next sweep need not
   int c0_valid;
@@ -426,6 +429,12 @@ int taps_fd_prepare_enqueue(taps_problem* P, int solver, int M, std::vector<FdPe
 int taps_fd_prepare_finish(std::vector<FdPending>* pend);
 int taps_lu_needs_tuning(const taps_problem* P, int solver, int M);
 int taps_check_status(int* d_status, cudaStream_t s);
+// Block-banded elimination from both ends (twosided.cu): CTAs per cluster for a dim (0:
+// the one-ended elimination), scratch, and the solve of an assembled system.
+int taps_ts_setup(int maxsm, int* most, size_t* smem);
+int taps_ts_ctas(const taps_problem* P, int hb, int M);
+size_t taps_ts_scratch_doubles(int hb, int M);
+int taps_ts_solve(taps_problem* P, taps_factors* U, int d, int nc);
 int taps_fd_eligible(const taps_problem* P, int d, int* slotA, int* slotB);
 int taps_fd_solve(taps_problem* P, taps_factors* U, int d, int precision);
 void taps_fd_release(taps_dim* dm);
