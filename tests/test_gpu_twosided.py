@@ -1,7 +1,7 @@
 """Block elimination from both ends against the FP64 oracle's banded solver, at the sizes
 where its pieces change: no, one and two eliminated nodes beside the middle, every band
 half-width, one and several columns per CTA, one and two row slots per lane (M = 32, 33),
-the largest M of the route at s = 2 (37) and one beyond it."""
+the largest M of the route at s = 2 (37); beyond it and for s > 2 the one-ended elimination."""
 import numpy as np
 import pytest
 
