@@ -792,6 +792,7 @@ extern "C" int taps_problem_copy_source(const taps_problem* P, int r, int d, dou
 extern "C" void taps_factors_destroy(taps_factors* U) {
   if (!U) return;
   for (int d = 0; d < TAPS_MAX_DIMS; ++d) cudaFree(U->d_U[d]);
+  cudaFree(U->d_ptab);
   delete U;
 }
 

@@ -6,6 +6,8 @@
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
+#include <mutex>
 #include <vector>
 
 #include "taps_internal.cuh"
@@ -700,10 +702,229 @@ __global__ void eval_points_kernel(PointDims PD, int D, int M, int n_pts, const 
   out[ip] = u;
 }
 
+// ---------------------------------------------------------------------------------
+// The same through per-element polynomials.  Inside an element every kernel of a patch is one
+// cubic (its breakpoints |x - x_j| = a h / 2 and a h fall on nodes or beyond the patch), so
+// with monomials up to p <= 3 and the linear hats the field of a mode is a polynomial of
+// degree 4 there.  Its coefficients come from the shape tables at the element's Gauss points:
+// the Legendre coefficients of a degree-4 polynomial are exact Gauss sums from 5 points on.
+// Per point, dim and mode 4 FMAs and a product remain instead of the patch functions (two per
+// element: splines, a division and two moment products each, ~300 FP64 instructions), which
+// were what a point cost: 65536 points in 8 dims at 8 modes 483 us, FP64 issue.
+// ---------------------------------------------------------------------------------
+#define EP_Q 5        // coefficients per element and mode
+#define EP_PAIRS 4    // mode pairs per pass over the dims
+struct EpBuild {
+  const double* N[TAPS_MAX_DIMS];   // [n - 1][nq][nloc]
+  const double* U[TAPS_MAX_DIMS];
+  double* tab[TAPS_MAX_DIMS];       // [n - 1][mode pair][EP_Q][2], in powers of 2 t - 1
+  double Q[TAPS_MAX_DIMS][EP_Q][TAPS_MAX_QUAD];   // Gauss point values to coefficients
+  int n[TAPS_MAX_DIMS], s[TAPS_MAX_DIMS], nq[TAPS_MAX_DIMS], nloc[TAPS_MAX_DIMS], off[TAPS_MAX_DIMS],
+      nf[TAPS_MAX_DIMS];
+};
+
+__global__ void __launch_bounds__(128) eval_points_table_kernel(const __grid_constant__ EpBuild B, int M) {
+  const int d = blockIdx.y, ne = B.n[d] - 1, mp = (M + 1) / 2;
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (long long)ne * mp * 2) return;
+  const int e = (int)(idx % ne), m = (int)(idx / ne);   // neighbouring threads: neighbouring nodes of a column
+  double c[EP_Q] = {};
+  if (m < M) {   // an odd count's last pair has a zero mode
+    const int nloc = B.nloc[d], nq = B.nq[d], f0 = e - B.s[d] - B.off[d];
+    const double* col = B.U[d] + (size_t)m * B.nf[d];
+    double u[2 * TAPS_MAX_S + 2];
+#pragma unroll
+    for (int k = 0; k < 2 * TAPS_MAX_S + 2; ++k) u[k] = (k < nloc && f0 + k >= 0 && f0 + k < B.nf[d]) ? col[f0 + k] : 0.0;
+    const double* N = B.N[d] + (size_t)e * nq * nloc;
+    for (int g = 0; g < nq; ++g) {
+      double v = 0.0;
+#pragma unroll
+      for (int k = 0; k < 2 * TAPS_MAX_S + 2; ++k)
+        if (k < nloc) v = fma(N[g * nloc + k], u[k], v);
+#pragma unroll
+      for (int q = 0; q < EP_Q; ++q) c[q] = fma(B.Q[d][q][g], v, c[q]);
+    }
+  }
+  double* out = B.tab[d] + ((size_t)e * mp + (m >> 1)) * (2 * EP_Q) + (m & 1);
+#pragma unroll
+  for (int q = 0; q < EP_Q; ++q) out[2 * q] = c[q];
+}
+
+struct EpDims {
+  const double* tab[TAPS_MAX_DIMS];
+  double lo[TAPS_MAX_DIMS], hi[TAPS_MAX_DIMS], step[TAPS_MAX_DIMS], inv[TAPS_MAX_DIMS];
+  int n[TAPS_MAX_DIMS];
+};
+
+template <int D>
+__global__ void __launch_bounds__(128) eval_points_poly_kernel(const __grid_constant__ EpDims E, int M, int n_pts,
+                                                               const double* __restrict__ pts,
+                                                               double* __restrict__ out) {
+  const int ip = blockIdx.x * blockDim.x + threadIdx.x;
+  if (ip >= n_pts) return;
+  const int mp = (M + 1) / 2;
+  double tau[D];
+  const double2* row[D];
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const double x = fmin(fmax(pts[(size_t)ip * D + d], E.lo[d]), E.hi[d]);
+    const int e = min(max((int)floor((x - E.lo[d]) * E.inv[d]), 0), E.n[d] - 2);
+    tau[d] = fma(2.0 * E.inv[d], x - fma((double)e, E.step[d], E.lo[d]), -1.0);
+    row[d] = reinterpret_cast<const double2*>(E.tab[d]) + (size_t)e * mp * EP_Q;
+  }
+  double u = 0.0;
+  for (int m0 = 0; m0 < mp; m0 += EP_PAIRS) {
+    double2 acc[EP_PAIRS];
+#pragma unroll
+    for (int j = 0; j < EP_PAIRS; ++j) acc[j] = make_double2(1.0, 1.0);
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      const double2* c = row[d] + (size_t)m0 * EP_Q;
+      const double t = tau[d];
+#pragma unroll
+      for (int j = 0; j < EP_PAIRS; ++j) {
+        if (m0 + j >= mp) break;
+        double2 v = __ldg(c + j * EP_Q + EP_Q - 1);
+#pragma unroll
+        for (int q = EP_Q - 2; q >= 0; --q) {
+          const double2 w = __ldg(c + j * EP_Q + q);
+          v.x = fma(v.x, t, w.x);
+          v.y = fma(v.y, t, w.y);
+        }
+        acc[j].x *= v.x;
+        acc[j].y *= v.y;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < EP_PAIRS; ++j) {
+      if (m0 + j >= mp) break;
+      u += acc[j].x;
+      if (2 * (m0 + j) + 1 < M) u += acc[j].y;
+    }
+  }
+  out[ip] = u;
+}
+
+// Whether every kernel of the dim's patches is a single cubic inside each element, and the
+// shape tables hold enough points for its products.
+static bool ep_polynomial(const taps_dim* dm) {
+  const double a = dm->desc.a;
+  auto on_node = [&](double r) { return r >= dm->desc.s + 1 || r == floor(r); };
+  return dm->nq >= EP_Q && on_node(0.5 * a) && on_node(a);
+}
+
+// Legendre coefficients (2 l + 1) sum_g w_g P_l(tau_g) f_g (weights on [0, 1]), then powers.
+static void ep_fit(const taps_dim* dm, double (*Q)[TAPS_MAX_QUAD]) {
+  static const double P[EP_Q][EP_Q] = {{1.0, 0.0, 0.0, 0.0, 0.0},
+                                       {0.0, 1.0, 0.0, 0.0, 0.0},
+                                       {-0.5, 0.0, 1.5, 0.0, 0.0},
+                                       {0.0, -1.5, 0.0, 2.5, 0.0},
+                                       {0.375, 0.0, -3.75, 0.0, 4.375}};
+  for (int g = 0; g < dm->nq; ++g) {
+    const double t = 2.0 * dm->gq_t[g] - 1.0;
+    for (int q = 0; q < EP_Q; ++q) Q[q][g] = 0.0;
+    for (int l = 0; l < EP_Q; ++l) {
+      double v = 0.0;
+      for (int q = EP_Q - 1; q >= 0; --q) v = v * t + P[l][q];
+      for (int q = 0; q < EP_Q; ++q) Q[q][g] += (2 * l + 1) * dm->gq_w[g] * v * P[l][q];
+    }
+  }
+}
+
+// The coefficient tables' memory of a factor set, sized for its mode capacity, made on first
+// use and kept until the factors go (every call fills it from the current factors).  Null when
+// it is not there and cannot be made now (a capture under way, no memory).
+static std::mutex g_ep_mutex;
+static double* ep_tables(const taps_problem* P, taps_factors* U) {
+  std::lock_guard<std::mutex> lock(g_ep_mutex);
+  if (U->d_ptab) return U->d_ptab;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(P->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  size_t tot = 0;
+  for (int d = 0; d < P->D; ++d) tot += (size_t)(P->dims[d]->n - 1) * ((U->M_cap + 1) / 2) * (2 * EP_Q);
+  double* p = nullptr;
+  if (taps_alloc((void**)&p, sizeof(double) * tot) != TAPS_OK) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  U->d_ptab = p;
+  return p;
+}
+
+// The polynomial route when it applies; *done = 0 leaves the call to eval_points_kernel.
+static int eval_points_poly(const taps_problem* P, taps_factors* U, int n_pts, const double* pts, double* out,
+                            int* done) {
+  *done = 0;
+  const int M = U->M, mp = (M + 1) / 2;
+  if (M < 1) return TAPS_OK;
+  long long elems = 0;
+  for (int d = 0; d < P->D; ++d) {
+    if (!ep_polynomial(P->dims[d])) return TAPS_OK;
+    elems += P->dims[d]->n - 1;
+  }
+  // An entry of the tables costs ~70 FMAs, a point without them ~300 + 2 M FP64 instructions
+  // per dim.  Few points of long dims with many modes stay on the other kernel, unless the
+  // tables are small against its latency (~5 us per dim however few the points; 32768 entries
+  // are 4 us).
+  if (elems * M > 32768LL * P->D && 70 * elems * M > (300LL + 2 * M) * n_pts * P->D) return TAPS_OK;
+  double* tab = ep_tables(P, U);
+  if (!tab) return TAPS_OK;
+  EpBuild B;
+  EpDims E;
+  memset(&B, 0, sizeof(B));
+  memset(&E, 0, sizeof(E));
+  int nmax = 0;
+  for (int d = 0; d < P->D; ++d) {
+    const taps_dim* dm = P->dims[d];
+    B.N[d] = dm->d_N;
+    B.U[d] = U->d_U[d];
+    B.tab[d] = tab;
+    ep_fit(dm, B.Q[d]);
+    B.n[d] = dm->n;
+    B.s[d] = dm->desc.s;
+    B.nq[d] = dm->nq;
+    B.nloc[d] = dm->nloc;
+    B.off[d] = dm->off;
+    B.nf[d] = dm->nf;
+    E.tab[d] = tab;
+    const DimParams q = make_params(dm);
+    E.lo[d] = q.lo;
+    E.hi[d] = q.hi;
+    E.step[d] = q.step;
+    E.inv[d] = 1.0 / q.step;
+    E.n[d] = dm->n;
+    nmax = std::max(nmax, dm->n - 1);
+    tab += (size_t)(dm->n - 1) * mp * (2 * EP_Q);
+  }
+  eval_points_table_kernel<<<dim3((unsigned)(((long long)nmax * mp * 2 + 127) / 128), P->D), 128, 0, P->stream>>>(B, M);
+  const unsigned grid = (n_pts + 127) / 128;
+  switch (P->D) {
+    case 1: eval_points_poly_kernel<1><<<grid, 128, 0, P->stream>>>(E, M, n_pts, pts, out); break;
+    case 2: eval_points_poly_kernel<2><<<grid, 128, 0, P->stream>>>(E, M, n_pts, pts, out); break;
+    case 3: eval_points_poly_kernel<3><<<grid, 128, 0, P->stream>>>(E, M, n_pts, pts, out); break;
+    case 4: eval_points_poly_kernel<4><<<grid, 128, 0, P->stream>>>(E, M, n_pts, pts, out); break;
+    case 5: eval_points_poly_kernel<5><<<grid, 128, 0, P->stream>>>(E, M, n_pts, pts, out); break;
+    case 6: eval_points_poly_kernel<6><<<grid, 128, 0, P->stream>>>(E, M, n_pts, pts, out); break;
+    case 7: eval_points_poly_kernel<7><<<grid, 128, 0, P->stream>>>(E, M, n_pts, pts, out); break;
+    default: eval_points_poly_kernel<8><<<grid, 128, 0, P->stream>>>(E, M, n_pts, pts, out); break;
+  }
+  TAPS_CUDA(cudaGetLastError());
+  *done = 1;
+  return TAPS_OK;
+}
+
 extern "C" int taps_eval_points(const taps_problem* prob, const taps_factors* U, int n_pts,
                                 const double* pts_dev, double* out_dev) {
   if (!prob || !U || n_pts < 0 || (n_pts > 0 && (!pts_dev || !out_dev))) return TAPS_ERR_INVALID_ARG;
   if (n_pts == 0) return TAPS_OK;
+  if (U->prob == prob) {
+    int done = 0;
+    TAPS_TRY(eval_points_poly(prob, const_cast<taps_factors*>(U), n_pts, pts_dev, out_dev, &done));
+    if (done) return TAPS_OK;
+  }
   PointDims PD;
   memset(&PD, 0, sizeof(PD));
   for (int d = 0; d < prob->D; ++d) {

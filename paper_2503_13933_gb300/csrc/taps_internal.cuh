@@ -191,6 +191,7 @@ struct taps_factors {
   const taps_problem* prob;
   int M, M_cap;
   double* d_U[TAPS_MAX_DIMS];  // [nf_d][M_cap] column-major, leading dim nf_d
+  double* d_ptab;              // element polynomials of taps_eval_points (made on first use)
 };
 
 // ---------------------------------------------------------------------------------
