@@ -868,87 +868,147 @@ __global__ void __launch_bounds__(128) fd_small_solve_quad_kernel(const double* 
 }
 
 // One CTA per node i (M > 32): solve (mu_i C_A + C_B) y = g_i by LU with partial
-// pivoting in shared memory, the right-hand side carried along as column M.  Per
-// step p, warp 0 finds the pivot row (largest magnitude, ties to the smaller row;
-// integer compares of the magnitudes' bit patterns), swaps it into place and takes the
-// pivot's reciprocal; then warp w updates the rows
-// r = p+1+w, p+5+w, ... (lanes over the columns c > p, coalesced) with one FMA per
-// entry, T[r][c] -= l_r T[p][c], l_r = T[r][p] / T[p][p] (as a product with the
-// reciprocal, seed plus refinement, formed by warp 0 for all rows at once).  The
-// trailing update is FP64 FMA issue on all four SM sub-partitions (eight warps, so that
-// two CTAs per SM keep four warps on each sub-partition); two barriers per step.  Back
-// substitution column by column: x_r = b_r U_rr^-1 (the kept reciprocal), then every
-// thread removes x_r from its rows' right-hand sides.  A zero or non-finite
-// pivot is reported as TAPS_DEV_SINGULAR.
-__global__ void __launch_bounds__(256) fd_small_solve_kernel(const double* __restrict__ CA,
-                                                             const double* __restrict__ CB,
-                                                             const double* __restrict__ mu,
-                                                             const double* __restrict__ G, int M,
-                                                             double* __restrict__ Y, int* status) {
+// pivoting in shared memory, the right-hand side carried along as column M.  A step's
+// pivot work is a chain of its own (search, reciprocal, multipliers: ~1200 clocks) beside
+// the trailing update's FP64 issue ((M - p)^2 / 2 clocks), so the two overlap: during step
+// p warp 0 updates column p + 1 first, finds its pivot row (largest magnitude, ties to the
+// smaller row; integer compares of the magnitudes' bit patterns), takes the reciprocal
+// (seed plus refinement) and forms the next step's multipliers l_r = T[r][p+1] / pivot with
+// the lanes over the rows, while warps 1 .. update the other columns, one FMA per entry,
+// T[r][c] -= l_r T[p][c], the threads dealt out over the whole trailing block so that no lane
+// idles at row ends.  Rows change places in a table of row offsets, not in memory, and a step
+// has one barrier.  Warp 0 then substitutes back alone, its lanes holding the right-hand
+// side, with the kept reciprocals.  A zero or non-finite pivot is reported as
+// TAPS_DEV_SINGULAR.  Every entry takes the same FMAs in the same order as with two barriers
+// per step and the pivot search between them.  1534 systems of 100 modes: 1.97 -> 1.32 ms
+// (0.85 ms of FP64 issue).
+#define FS_THREADS 256
+__global__ void __launch_bounds__(FS_THREADS, 2) fd_small_solve_kernel(const double* __restrict__ CA,
+                                                                       const double* __restrict__ CB,
+                                                                       const double* __restrict__ mu,
+                                                                       const double* __restrict__ G, int M,
+                                                                       double* __restrict__ Y, int* status) {
   extern __shared__ double T[];   // [M][M+1]: matrix | rhs
-  __shared__ double invd[TAPS_MAX_M];   // reciprocals of the pivots
-  __shared__ double lmul[TAPS_MAX_M];   // the step's multipliers, by row
-  __shared__ int bad;
-  const int i = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+  __shared__ double invd[TAPS_MAX_M];      // reciprocals of the pivots
+  __shared__ double lmul[2][TAPS_MAX_M];   // multipliers of two steps, by logical row
+  __shared__ int rowat[2][TAPS_MAX_M];     // offset of row r in T, for two steps (rows from the step's on)
+  __shared__ int rowfin[TAPS_MAX_M];       // offsets of the pivot rows
+  const int i = blockIdx.x, tid = threadIdx.x;
+  const int lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int ld = M + 1;
   const double mi = mu ? mu[i] : 0.0;
-  for (int idx = tid; idx < M * M; idx += nt) {
+  for (int idx = tid; idx < M * M; idx += FS_THREADS) {
     int r = idx / M, c = idx % M;
     T[r * ld + c] = (CA ? mi * CA[idx] : 0.0) + CB[idx];
   }
-  for (int r = tid; r < M; r += nt) T[r * ld + M] = G[(size_t)i * M + r];
-  if (tid == 0) bad = 0;
+  for (int r = tid; r < M; r += FS_THREADS) {
+    T[r * ld + M] = G[(size_t)i * M + r];
+    rowat[0][r] = r * ld;
+  }
   __syncthreads();
-  for (int p = 0; p < M; ++p) {
-    if (warp == 0) {   // argmax |T[r][p]|, r >= p (ties to the smaller r), swap, reciprocal
-      // compared as the bit patterns of |T[r][p]| (non-negative doubles order like
-      // their bits): integer compares, off the FP64 pipe the update warps keep busy
-      long long best = -1;
-      int br = p;
-      for (int r = p + lane; r < M; r += 32) {
-        const long long a = __double_as_longlong(fabs(T[r * ld + p]));
+  // warp 0: the pivot of step p, whose column is final in T; rows in `at` order on entry,
+  // `to` receives the step's order and `l` its multipliers
+  bool bad = false;
+  auto pivot = [&](int p, const int* at, int* to, double* l) {
+    constexpr int S = TAPS_MAX_M / 32;
+    double v[S];
+    long long best = -1;
+    int br = p;
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      const int r = p + lane + 32 * s;
+      if (r < M) {
+        v[s] = T[at[r] + p];
+        const long long a = __double_as_longlong(fabs(v[s]));
         if (a > best) { best = a; br = r; }
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int orr = __shfl_xor_sync(0xffffffffu, br, o);
-        if (ob > best || (ob == best && orr < br)) { best = ob; br = orr; }
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int orr = __shfl_xor_sync(0xffffffffu, br, o);
+      if (ob > best || (ob == best && orr < br)) { best = ob; br = orr; }
+    }
+    const double pv = T[at[br] + p];
+    const bool ok = taps_finite_nonzero(pv);
+    const double inv = ok ? taps_rcp(pv) : 0.0;
+    bad |= !ok;
+    if (lane == 0) {
+      invd[p] = inv;
+      rowfin[p] = at[br];
+    }
+    const double v0 = T[at[p] + p];   // the row that takes br's place
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      const int r = p + lane + 32 * s;
+      if (r < M) {
+        to[r] = at[r == p ? br : (r == br ? p : r)];
+        if (r > p) l[r] = (r == br ? v0 : v[s]) * inv;
       }
-      if (br != p)
-        for (int c = p + lane; c <= M; c += 32) {
-          const double t = T[p * ld + c];
-          T[p * ld + c] = T[br * ld + c];
-          T[br * ld + c] = t;
+    }
+  };
+  if (warp == 0) pivot(0, rowat[0], rowat[1], lmul[0]);
+  __syncthreads();
+  for (int p = 0; p < M; ++p) {
+    const int* at = rowat[(p + 1) & 1];   // the order of step p
+    const double* l = lmul[p & 1];
+    const double* prow = T + rowfin[p];
+    if (warp == 0) {
+      if (p + 1 < M) {
+        const double pc = prow[p + 1];
+        for (int r = p + 1 + lane; r < M; r += 32) {
+          double* x = T + at[r] + p + 1;
+          *x = fma(-l[r], pc, *x);
         }
-      __syncwarp();
-      const double pv = T[p * ld + p];
-      const bool ok = taps_finite_nonzero(pv);
-      const double inv = ok ? taps_rcp(pv) : 0.0;
-      if (lane == 0) {
-        invd[p] = inv;
-        if (!ok) bad = 1;
+        __syncwarp();
+        pivot(p + 1, at, rowat[p & 1], lmul[(p + 1) & 1]);
       }
-      // the multipliers of every row below, lanes over rows: one FP64 instruction per
-      // 32 rows instead of one per row in the update warps
-      for (int r = p + 1 + lane; r < M; r += 32) lmul[r] = T[r * ld + p] * inv;
-    }
-    __syncthreads();
-    for (int r = p + 1 + warp; r < M; r += nw) {
-      const double l = lmul[r];
-      for (int c = p + 1 + lane; c <= M; c += 32) T[r * ld + c] = fma(-l, T[p * ld + c], T[r * ld + c]);
+    } else {
+      // columns p + 2 .. M of the rows after p, over warps 1 ..
+      const int w = M - 1 - p, rows = M - 1 - p;   // (the right-hand side among the columns)
+      if (w > 0) {
+        const int t = tid - 32, nt = FS_THREADS - 32;
+        int r = t / w, c = t - r * w;
+        const int dr = nt / w, dc = nt - dr * w;
+        while (r < rows) {
+          double* x = T + at[p + 1 + r] + p + 2 + c;
+          *x = fma(-l[p + 1 + r], prow[p + 2 + c], *x);
+          r += dr;
+          c += dc;
+          if (c >= w) {
+            c -= w;
+            ++r;
+          }
+        }
+      }
     }
     __syncthreads();
   }
-  for (int r = M - 1; r >= 0; --r) {
-    if (tid == 0) T[r * ld + M] *= invd[r];   // the kept reciprocal (0 for a bad pivot)
-    __syncthreads();
-    const double xr = T[r * ld + M];
-    for (int k = tid; k < r; k += nt) T[k * ld + M] = fma(-T[k * ld + r], xr, T[k * ld + M]);
-    __syncthreads();
+  if (warp != 0) return;
+  // x_r in the lane that holds row r
+  const int* at = rowfin;
+  constexpr int S = TAPS_MAX_M / 32;
+  double b[S];
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const int r = lane + 32 * s;
+    b[s] = r < M ? T[at[r] + M] : 0.0;
   }
-  for (int r = tid; r < M; r += nt) Y[(size_t)i * M + r] = T[r * ld + M];
-  if (tid == 0 && bad) taps_flag(status, TAPS_DEV_SINGULAR);
+#pragma unroll
+  for (int sr = S - 1; sr >= 0; --sr) {
+    for (int r = min(M - 1, 32 * sr + 31); r >= 32 * sr; --r) {
+      const double xr = __shfl_sync(0xffffffffu, b[sr], r & 31) * invd[r];   // 0 for a bad pivot
+      if (lane == (r & 31)) b[sr] = xr;
+#pragma unroll
+      for (int s = 0; s <= sr; ++s) {
+        const int k = lane + 32 * s;
+        if (k < r) b[s] = fma(-T[at[k] + r], xr, b[s]);
+      }
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < S; ++s)
+    if (lane + 32 * s < M) Y[(size_t)i * M + lane + 32 * s] = b[s];
+  if (bad && lane == 0) taps_flag(status, TAPS_DEV_SINGULAR);
 }
 
 // ---------------------------------------------------------------------------------
@@ -1235,7 +1295,7 @@ int taps_fd_solve(taps_problem* P, taps_factors* U, int d, int precision) {
         TAPS_TRY(taps_allow_dyn_smem((const void*)fd_small_solve_kernel, maxsm));
         smem_ok = true;
       }
-      fd_small_solve_kernel<<<n, 256, sizeof(double) * (size_t)M * (M + 1), s>>>(
+      fd_small_solve_kernel<<<n, FS_THREADS, sizeof(double) * (size_t)M * (M + 1), s>>>(
           CA, CB, slotA >= 0 ? E->mu : nullptr, G, M, Y, P->d_status);
     }
     ++launches;
