@@ -372,9 +372,13 @@ __device__ __forceinline__ void ts_eliminate(const TsArgs& a, int base, int dir,
           double* x = column(ci) + ring_row(r);
           const double* p = pan + M + r;   // row r of the following nodes
           const double* wv = wbuf + ci * M;
-          double t0 = *x;
+          // the products' sum first, one subtraction after: a chain that starts from the entry
+          // rounds at the entry's size in every term (2 - 3 times the error on ill-conditioned
+          // systems)
+          double sum = 0.0;
 #pragma unroll 4
-          for (int l = 0; l < M; ++l, p += rows) t0 = fma(-p[0], wv[l], t0);
+          for (int l = 0; l < M; ++l, p += rows) sum = fma(p[0], wv[l], sum);
+          const double t0 = *x - sum;
           if (e < npush) {
             double* dst = npan + (size_t)(g0 + (ci << sh) - lo) * rows + r;
             for (unsigned t = 0; t < nc; ++t) *cluster.map_shared_rank(dst, t) = t0;
