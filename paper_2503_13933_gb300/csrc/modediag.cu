@@ -16,11 +16,10 @@
 //                    Cholesky C_X = L L^T, S = L^-1 C_Y L^-T, cyclic Jacobi
 //                    S = Q diag(lam) Q^T, W = P L^-T Q, and Wc_r = W^T c_r for the
 //                    right-hand side F W = sum_r q_r (W^T c_r)^T.
-//   md_prep_kernel   every system's band rows Op_X + lam_j Op_Y and right-hand side,
-//                    in parallel over rows, band entries and systems.
-//   md_band_kernel   thread j: Gaussian elimination without pivoting of the banded
-//                    system (half-bandwidth HB) with the active rows in a register
-//                    ring, then back substitution; Z is n_d x M row-major.
+//   md_rhs_kernel    every system's right-hand side (F W)_j.
+//   md_band_kernel   warp j: Gaussian elimination without pivoting of the banded system
+//                    Op_X + lam_j Op_Y (half-bandwidth HB), the lanes sharing a step,
+//                    then back substitution; Z is n_d x M row-major.
 //   md_out_kernel    U = Z W^T into the factor layout, the old factor into Save.
 //
 // The eliminations need no pivoting: with X the mass-like operator (symmetric
@@ -1296,133 +1295,149 @@ __global__ void md_cw_kernel(const double* __restrict__ c, const double* __restr
   cw[idx] = s;
 }
 
-// Padding rows below the matrix (identity rows, zero right-hand side) let the
-// elimination run whole unrolled groups and read ahead without bounds tests.
-#define MD_PAD 24
-
-// Ab[(i * (2HB+2) + k) * M + j]: row i of Op_X + lam_j Op_Y in band-relative form
-// (k = column - i + HB, zero outside the matrix) and, at k = 2HB+1, the right-hand side
-// (F W)[i][j] = sum_r q_r[i] Wc_r[j]; rows n .. n+MD_PAD-1 are identity rows.
-template <int HB>
-__global__ void md_prep_kernel(const double* __restrict__ bx, const double* __restrict__ by,
-                               const double* __restrict__ lam, const double* __restrict__ q,
-                               const double* __restrict__ cw, int Rf, int n, int M, double* __restrict__ Ab) {
-  constexpr int W2 = 2 * HB + 1, RW = W2 + 1;
+// Fw[i][j] = (F W)[i][j] = sum_r q_r[i] Wc_r[j], one FMA chain per entry; the next sixteen terms
+// are loaded while sixteen are added (a moving source has hundreds).
+__global__ void md_rhs_kernel(const double* __restrict__ q, const double* __restrict__ cw, int Rf, int n, int M,
+                              double* __restrict__ Fw) {
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long tot = (long long)(n + MD_PAD) * RW * M;
-  if (idx >= tot) return;
-  const int j = (int)(idx % M);
-  const int k = (int)((idx / M) % RW);
-  const int i = (int)(idx / ((long long)M * RW));
-  double v = 0.0;
-  if (i >= n) {
-    v = (k == HB) ? 1.0 : 0.0;
-  } else if (k < W2) {
-    const int col = i + k - HB;
-    if (col >= 0 && col < n) v = fma(lam[j], by[(size_t)i * W2 + k], bx[(size_t)i * W2 + k]);
-  } else {
-    for (int r = 0; r < Rf; ++r) v = fma(q[(size_t)r * n + i], cw[r * M + j], v);
+  if (idx >= (long long)n * M) return;
+  const int j = (int)(idx % M), i = (int)(idx / M);
+  constexpr int T = 16;
+  double a[2][T], b[2][T], v = 0.0;
+  auto load = [&](int r0, double* x, double* y) {
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+      x[t] = r0 + t < Rf ? q[(size_t)(r0 + t) * n + i] : 0.0;
+      y[t] = r0 + t < Rf ? cw[(size_t)(r0 + t) * M + j] : 0.0;
+    }
+  };
+  auto add = [&](int r0, const double* x, const double* y) {
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+      if (r0 + t < Rf) v = fma(x[t], y[t], v);
+  };
+  load(0, a[0], b[0]);
+  for (int r0 = 0; r0 < Rf; r0 += 2 * T) {
+    load(r0 + T, a[1], b[1]);
+    add(r0, a[0], b[0]);
+    load(r0 + 2 * T, a[0], b[0]);
+    add(r0 + T, a[1], b[1]);
   }
-  Ab[idx] = v;
+  Fw[idx] = v;
 }
 
-// Thread j < M solves (Op_X + lam_j Op_Y) z_j = (F W)_j by Gaussian elimination without
-// pivoting (no fill outside the band).  The active rows i .. i+HB live in a ring of
-// NS = HB+1 register rows in band-relative form, so a row keeps its storage while the
-// window moves: row i+r sits in slot (i+r) mod NS, its entry in column i + c at
-// HB + c - r.  The loop is unrolled by U = lcm(NS, 2) so that every slot index is a
-// compile-time constant; the row entering at step i (row i+HB+1, into the pivot's slot)
-// was loaded two steps earlier.  Stored per step: the pivot row scaled by the pivot's
-// reciprocal, scratch[(i * (HB+1) + c) * M + j] (c = 0: right-hand side, 1..HB:
-// superdiagonal); back substitution walks them upwards with the same ring.
+// Warp j solves (Op_X + lam_j Op_Y) z_j = (F W)_j by Gaussian elimination without pivoting (no
+// fill outside the band).  An FP64 instruction costs its sub-partition ~64 clocks whatever its
+// active lanes, so the lanes share one system's step (one thread per system: 45 instructions a
+// step, 2900 clocks; here 7, ~500): lane (r, c), 1 <= r <= HB, 1 <= c <= HB + 1, holds entry
+// (i + r, i + c) of the window below pivot i (c = HB + 1: the right-hand side).  For the next
+// pivot the window moves one row and column by shuffles; its last row and column are the
+// band's own entries Op_X + lam_j Op_Y, formed from loads issued four steps earlier, as are
+// the pivot row's last entry and the pivot column's (the two lanes after the window's).  Per
+// step the pivot row scaled by the pivot's reciprocal is kept (scratch[j][i][HB + 1], 0: the
+// right-hand side).  Back substitution pushes each z_i into the rows above, lane c - 1 holding
+// row i - c.  Every entry takes the operations of the thread-per-system form in their order.
+// 510 nodes, 31 systems: 936 -> 255 us.
 template <int HB>
-__global__ void __launch_bounds__(32) md_band_kernel(const double* __restrict__ Ab, int n, int M,
-                                                     double* __restrict__ scratch, double* __restrict__ Z,
-                                                     int* status) {
-  constexpr int W2 = 2 * HB + 1, RW = W2 + 1, NS = HB + 1;
-  constexpr int U = (NS % 2 == 0) ? NS : 2 * NS;
-  const int j = blockIdx.x * 32 + threadIdx.x;   // system index (one warp per 32 systems)
-  if (j >= M) return;
-  const int nsteps = ((n + U - 1) / U) * U;   // <= n + U - 1; rows read <= nsteps + HB + 2
-  double A[NS][W2];
-  double b[NS];
-#pragma unroll
-  for (int r = 0; r < NS; ++r) {
-    const double* row = Ab + (size_t)r * RW * M + j;
-#pragma unroll
-    for (int k = 0; k < W2; ++k) A[r][k] = row[(size_t)k * M];
-    b[r] = row[(size_t)W2 * M];
+__global__ void __launch_bounds__(32) md_band_kernel(const double* __restrict__ bx, const double* __restrict__ by,
+                                                     const double* __restrict__ lam, const double* __restrict__ Fw,
+                                                     int n, int M, double* __restrict__ scratch,
+                                                     double* __restrict__ Z, int* status) {
+  constexpr int W2 = 2 * HB + 1, NS = HB + 1, NC = HB + 1, GRID = HB * NC, AHEAD = 4;
+  constexpr unsigned ALL = 0xffffffffu;
+  const int j = blockIdx.x, lane = threadIdx.x;
+  const double lj = lam[j];
+  const bool in_window = lane < GRID;
+  const int r = in_window ? lane / NC + 1 : 1, c = in_window ? lane % NC + 1 : 1;
+  auto at = [](int rr, int cc) { return (rr - 1) * NC + (cc - 1); };
+  // where this lane's operands of a step are: its entry, the pivot row's in its column, the
+  // pivot column's in its row
+  const bool enters = in_window && ((r == HB) || (c == HB));
+  const int src_mine = enters || !in_window ? lane : at(r + 1, c < HB ? c + 1 : NC);
+  const int src_u = c < HB ? at(1, c + 1) : (c == HB ? GRID : at(1, NC));
+  const int src_c = r < HB ? at(r + 1, 1) : GRID + 1;
+  // the band's entry (or right-hand side) that enters at step i for this lane: row i + rofs
+  const bool loads = enters || lane == GRID || lane == GRID + 1;
+  const bool is_rhs = in_window && c == NC;
+  const int rofs = lane == GRID ? 0 : (lane == GRID + 1 ? HB : r);
+  const int kk = lane == GRID ? 2 * HB : (lane == GRID + 1 ? 0 : c - r + HB);
+  auto entry = [&](int row, int k, bool rhs, double& x, double& y) {   // value = x + lam_j y
+    x = y = 0.0;
+    if (row >= n) {   // below the matrix: the identity
+      x = (!rhs && k == HB) ? 1.0 : 0.0;
+    } else if (rhs) {
+      x = Fw[(size_t)row * M + j];
+    } else if (row + k - HB >= 0 && row + k - HB < n) {
+      x = bx[(size_t)row * W2 + k];
+      y = by[(size_t)row * W2 + k];
+    }
+  };
+  double W = 0.0, px[AHEAD], py[AHEAD];
+  if (in_window) {   // entry (r - 1, c - 1): the window below a pivot before the first
+    double x, y;
+    entry(r - 1, c - r + HB, is_rhs, x, y);
+    W = fma(lj, y, x);
   }
-  double st[2][RW];   // staged rows: row i+HB+1 enters at step i from st[i & 1]
 #pragma unroll
-  for (int t = 0; t < 2; ++t) {
-    const double* row = Ab + (size_t)(HB + 1 + t) * RW * M + j;
-#pragma unroll
-    for (int k = 0; k < RW; ++k) st[t][k] = row[(size_t)k * M];
+  for (int t = 0; t < AHEAD; ++t) {
+    px[t] = py[t] = 0.0;
+    if (loads) entry(t + rofs, kk, is_rhs, px[t], py[t]);
   }
+  double* rows = scratch + (size_t)j * n * NS;
+  const int out_slot = c == NC ? 0 : c;
+  const bool writes = in_window && r == 1;
   bool bad = false;
-  for (int i0 = 0; i0 < nsteps; i0 += U) {
+  for (int i0 = 0; i0 < n; i0 += AHEAD) {
 #pragma unroll
-    for (int ph = 0; ph < U; ++ph) {
-      const int i = i0 + ph;
-      const int P = ph % NS;
-      const double piv = A[P][HB];
-      const bool ok = fabs(piv) > 0.0 && isfinite(piv);
+    for (int t = 0; t < AHEAD; ++t) {
+      const int i = i0 + t;
+      if (i >= n) break;
+      const double raw = fma(lj, py[t], px[t]);
+      if (loads) entry(i + AHEAD + rofs, kk, is_rhs, px[t], py[t]);
+      const double X = in_window ? W : raw;
+      const double piv = __shfl_sync(ALL, X, at(1, 1));
+      const double u = __shfl_sync(ALL, X, src_u);
+      const double cr = __shfl_sync(ALL, X, src_c);
+      const double moved = __shfl_sync(ALL, X, src_mine);
+      const bool ok = taps_finite_nonzero(piv);
       bad |= !ok;
       const double inv = ok ? taps_rcp(piv) : 0.0;
-#pragma unroll
-      for (int r = 1; r <= HB; ++r) {
-        const int R = (ph + r) % NS;
-        const double l = A[R][HB - r] * inv;
-#pragma unroll
-        for (int c = 1; c <= HB; ++c) A[R][HB + c - r] -= l * A[P][HB + c];
-        b[R] -= l * b[P];
-      }
-      double* out = scratch + (size_t)i * NS * M + j;
-      out[0] = b[P] * inv;
-#pragma unroll
-      for (int c = 1; c <= HB; ++c) out[(size_t)c * M] = A[P][HB + c] * inv;
-      // row i+HB+1 takes the pivot's slot; row i+HB+3 is staged in its place
-      const int t = ph & 1;
-#pragma unroll
-      for (int k = 0; k < W2; ++k) A[P][k] = st[t][k];
-      b[P] = st[t][W2];
-      const double* row = Ab + (size_t)(i + HB + 3) * RW * M + j;
-#pragma unroll
-      for (int k = 0; k < RW; ++k) st[t][k] = row[(size_t)k * M];
+      const double l = cr * inv;
+      W = fma(-l, u, enters ? raw : moved);
+      if (writes) rows[(size_t)i * NS + out_slot] = u * inv;
     }
   }
-  if (bad) taps_flag(status, TAPS_DEV_SINGULAR);
-  // back substitution over the padded rows (their solution is zero): z_i = y_i -
-  // sum_c u_ic z_{i+c}, z in a ring of NS slots, stored rows loaded two steps ahead
-  double z[NS];
+  if (bad && lane == 0) taps_flag(status, TAPS_DEV_SINGULAR);
+  __syncwarp();   // the kept rows are read back by other lanes
+  // lane l < HB: the sum of row i - 1 - l so far, and its coefficient of z_i; lane HB: the
+  // right-hand side that enters there next
+  auto coef = [&](int i) {
+    const int row = i - 1 - lane;
+    return (lane < HB && row >= 0) ? rows[(size_t)row * NS + lane + 1] : 0.0;
+  };
+  auto next_y = [&](int i) {
+    const int row = i - 1 - HB;
+    return (lane == HB && row >= 0) ? rows[(size_t)row * NS] : 0.0;
+  };
+  double acc = (lane < HB && n - 2 - lane >= 0) ? rows[(size_t)(n - 2 - lane) * NS] : 0.0;
+  double z = rows[(size_t)(n - 1) * NS];
+  double pu[AHEAD], pv[AHEAD];
 #pragma unroll
-  for (int r = 0; r < NS; ++r) z[r] = 0.0;
-  double sr[2][NS];
-#pragma unroll
-  for (int t = 0; t < 2; ++t) {
-    const double* u = scratch + (size_t)(nsteps - 1 - t) * NS * M + j;
-#pragma unroll
-    for (int c = 0; c < NS; ++c) sr[t][c] = u[(size_t)c * M];
+  for (int t = 0; t < AHEAD; ++t) {
+    pu[t] = coef(n - 1 - t);
+    pv[t] = next_y(n - 1 - t);
   }
-  for (int i0 = nsteps - U; i0 >= 0; i0 -= U) {
+  for (int i0 = n - 1; i0 >= 0; i0 -= AHEAD) {
 #pragma unroll
-    for (int ph = U - 1; ph >= 0; --ph) {
-      const int i = i0 + ph;
-      const int t = (U - 1 - ph) & 1;   // rows nsteps-1, nsteps-2, ... alternate buffers
-      // the terms of z_{i+2} .. z_{i+HB} first: only the last FMA waits for z_{i+1}
-      double s = sr[t][0];
-#pragma unroll
-      for (int c = HB; c >= 2; --c) s -= sr[t][c] * z[(ph + c) % NS];
-      s -= sr[t][1] * z[(ph + 1) % NS];
-      z[ph % NS] = s;
-      if (i < n) Z[(size_t)i * M + j] = s;
-      const int nx = i - 2;
-      if (nx >= 0) {
-        const double* u = scratch + (size_t)nx * NS * M + j;
-#pragma unroll
-        for (int c = 0; c < NS; ++c) sr[t][c] = u[(size_t)c * M];
-      }
+    for (int t = 0; t < AHEAD; ++t) {
+      const int i = i0 - t;
+      if (i < 0) break;
+      if (lane == 0) Z[(size_t)i * M + j] = z;
+      acc = fma(-pu[t], z, lane == HB ? pv[t] : acc);
+      pu[t] = coef(i - AHEAD);
+      pv[t] = next_y(i - AHEAD);
+      z = __shfl_sync(ALL, acc, 0);
+      acc = __shfl_down_sync(ALL, acc, 1);
     }
   }
 }
@@ -1488,11 +1503,11 @@ int taps_dim_route(const taps_problem* P, int d, int solver, int M) {
 }
 
 // [TAPS_MAX_DIMS][M][M] bases, TAPS_MAX_DIMS ints (one double each), lam [M], W^T c
-// [Rf][M], Z [nf_max][M], eliminated rows [nf_max + MD_PAD][MD_MAX_HB + 1][M], band
-// rows [nf_max + MD_PAD][2 MD_MAX_HB + 2][M].  The caller zeroes it (no valid basis).
+// [Rf][M], Z [nf_max][M], eliminated rows [M][nf_max][MD_MAX_HB + 1], right-hand sides
+// [nf_max][M].  The caller zeroes it (no valid basis).
 size_t taps_md_scratch_doubles(int nf_max, int M, int Rf) {
   return (size_t)TAPS_MAX_DIMS * M * M + TAPS_MAX_DIMS + M + (size_t)Rf * M + (size_t)nf_max * M +
-         (size_t)(nf_max + MD_PAD) * (MD_MAX_HB + 1) * M + (size_t)(nf_max + MD_PAD) * (2 * MD_MAX_HB + 2) * M +
+         (size_t)nf_max * (MD_MAX_HB + 1) * M + (size_t)nf_max * M +
          (M > 32 ? (size_t)14 * M * M + 8 : 0);
 }
 
@@ -1527,11 +1542,10 @@ int taps_md_setup(int maxsm) {
 
 template <int HB>
 static cudaError_t md_band_launch(const double* bx, const double* by, const double* lam, const double* q,
-                                  const double* cw, int Rf, int n, int M, double* Ab, double* scratch, double* Z,
+                                  const double* cw, int Rf, int n, int M, double* Fw, double* scratch, double* Z,
                                   int* status, cudaStream_t s) {
-  const long long tot = (long long)(n + MD_PAD) * (2 * HB + 2) * M;
-  md_prep_kernel<HB><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(bx, by, lam, q, cw, Rf, n, M, Ab);
-  md_band_kernel<HB><<<(unsigned)((M + 31) / 32), 32, 0, s>>>(Ab, n, M, scratch, Z, status);
+  md_rhs_kernel<<<(unsigned)(((long long)n * M + 127) / 128), 128, 0, s>>>(q, cw, Rf, n, M, Fw);
+  md_band_kernel<HB><<<M, 32, 0, s>>>(bx, by, lam, Fw, n, M, scratch, Z, status);
   return cudaGetLastError();
 }
 
@@ -1617,7 +1631,7 @@ int taps_md_solve(taps_problem* P, taps_factors* U, int d) {
   double* cw = lam + M;
   double* Z = cw + (size_t)Rf * M;
   double* scratch = Z + (size_t)P->nf_max * M;
-  double* Ab = scratch + (size_t)(P->nf_max + MD_PAD) * (MD_MAX_HB + 1) * M;
+  double* Fw = scratch + (size_t)P->nf_max * (MD_MAX_HB + 1) * M;
   const size_t bsz = (size_t)n * dm->nb;
   const double* bx = dm->d_band + (size_t)P->ops[d][sx] * bsz;
   const double* by = sy >= 0 ? dm->d_band + (size_t)P->ops[d][sy] * bsz : bx;   // lam = 0 without Y
@@ -1626,8 +1640,8 @@ int taps_md_solve(taps_problem* P, taps_factors* U, int d) {
     md_eig_kernel<<<1, MD_THREADS, 0, s>>>(P->d_C + (size_t)sx * MM, sy >= 0 ? P->d_C + (size_t)sy * MM : nullptr,
                                             P->d_c, Rf, M, Wm, wM, lam, cw, P->d_status);
   } else {
-    // the eigen-solve's workspace follows the band rows (sized for M > 32 only)
-    double* gw = Ab + (size_t)(P->nf_max + MD_PAD) * (2 * MD_MAX_HB + 2) * M;
+    // the eigen-solve's workspace follows the right-hand sides (sized for M > 32 only)
+    double* gw = Fw + (size_t)P->nf_max * M;
     const int Np = M + (M & 1);
     const size_t smem_s = sizeof(double) * (size_t)Np * (Np + 1);   // opted in by taps_md_setup
     const size_t smem_sv = smem_s + sizeof(double) * (size_t)M * M;
@@ -1647,11 +1661,11 @@ int taps_md_solve(taps_problem* P, taps_factors* U, int d) {
   }
   cudaError_t ce = cudaSuccess;
   switch (hb) {
-    case 1: ce = md_band_launch<1>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Ab, scratch, Z, P->d_status, s); break;
-    case 2: ce = md_band_launch<2>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Ab, scratch, Z, P->d_status, s); break;
-    case 3: ce = md_band_launch<3>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Ab, scratch, Z, P->d_status, s); break;
-    case 4: ce = md_band_launch<4>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Ab, scratch, Z, P->d_status, s); break;
-    default: ce = md_band_launch<5>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Ab, scratch, Z, P->d_status, s); break;
+    case 1: ce = md_band_launch<1>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, s); break;
+    case 2: ce = md_band_launch<2>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, s); break;
+    case 3: ce = md_band_launch<3>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, s); break;
+    case 4: ce = md_band_launch<4>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, s); break;
+    default: ce = md_band_launch<5>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, s); break;
   }
   TAPS_CUDA(ce);
   const long long nM = (long long)n * M;
