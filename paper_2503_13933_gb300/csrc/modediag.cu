@@ -33,7 +33,7 @@
 
 #include "taps_internal.cuh"
 
-#define MD_THREADS 128
+#define MD_THREADS 512   // an entry of a round's updates per thread up to 32 modes
 #define MD_MAX_HB 5
 #define MD_MAX_SWEEPS 24
 
@@ -49,6 +49,149 @@ __device__ __forceinline__ void md_mm(double (*C)[33], const double (*A)[33], co
       for (int k = 0; k < M; ++k) s += A[i][k] * B[k][j];
     C[i][j] = s;
   }
+}
+
+// X <- L^-1 X for M x M shared-memory matrices: a step finishes row j and takes it from every
+// row below (all threads), so the chain is M steps instead of a thread's M^2 / 2 FMAs.  Each
+// entry's terms come in increasing j.
+__device__ __forceinline__ void md_lsolve(double (*X)[33], const double (*L)[33], const double* linv, int M) {
+  for (int j = 0; j < M; ++j) {
+    if ((int)threadIdx.x < M) X[j][threadIdx.x] *= linv[j];
+    __syncthreads();
+    const int cnt = (M - 1 - j) * M;
+    for (int idx = threadIdx.x; idx < cnt; idx += blockDim.x) {
+      const int i = j + 1 + idx / M, c = idx % M;
+      X[i][c] = fma(-L[i][j], X[j][c], X[i][c]);
+    }
+    __syncthreads();
+  }
+}
+
+// Rotations of S in FP32 as the seed of the FP64 ones: FP64 rounds are FP64 issue and a chain
+// of square roots and reciprocals (~5000 clocks each), FP32 rounds a twentieth of that, and
+// from a seed at FP32 accuracy the FP64 Jacobi sweeps have one or two left instead of seven or
+// more.  The seed basis Q is made orthonormal to FP64 by the series of (Q^T Q)^-1/2 up to the
+// square of E = I - Q^T Q (|E| ~ 1e-6), V <- Q and S <- Q^T S Q.  T and X: M x M scratch.
+// Returns false, with S and V as they were, if there is nothing to rotate at FP32 accuracy or
+// S is not finite.
+__device__ __forceinline__ bool md_seed_rotations(double (*S)[33], double (*V)[33], double (*T)[33],
+                                                  double (*X)[33], int M) {
+  __shared__ int top, any, turned;
+  __shared__ float fc[16], fs[16];
+  __shared__ int fp[16], fq[16];
+  float (*Sf)[33] = reinterpret_cast<float (*)[33]>(&T[0][0]);
+  float (*Vf)[33] = reinterpret_cast<float (*)[33]>(reinterpret_cast<float*>(&T[0][0]) + 32 * 33);
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int N = M + (M & 1), half = N / 2;
+  if (tid == 0) {
+    top = 0;
+    any = 0;
+  }
+  __syncthreads();
+  // the largest exponent: S scaled by a power of two into the range of FP32
+  for (int idx = tid; idx < M * M; idx += nt)
+    atomicMax(&top, __double2hiint(S[idx / M][idx % M]) & 0x7ff00000);
+  __syncthreads();
+  const int e = top >> 20;
+  if (e == 0 || e == 0x7ff || M < 2) return false;
+  const double scale = ldexp(1.0, 1023 - e);
+  for (int idx = tid; idx < N * N; idx += nt) {
+    const int i = idx / N, j = idx % N;
+    Sf[i][j] = (i < M && j < M) ? (float)(S[i][j] * scale) : 0.f;
+    Vf[i][j] = i == j ? 1.f : 0.f;
+  }
+  __syncthreads();
+  // the thread's block of S and entry pair of V, the same in every round (half^2 and half M
+  // are at most the block's 512 threads)
+  const int bk = tid / half, bl = tid % half, vl = tid / M, vi = tid % M;
+  for (int sw = 0; sw < 10; ++sw) {
+    if (tid == 0) turned = 0;
+    __syncthreads();
+    for (int r = 0; r < N - 1; ++r) {
+      if (tid < half) {
+        int a = tid == 0 ? r : r + tid, b = tid == 0 ? N - 1 : r - tid + N - 1;
+        if (tid > 0 && a >= N - 1) a -= N - 1;
+        if (tid > 0 && b >= N - 1) b -= N - 1;
+        const int p = min(a, b), q = max(a, b);
+        float c = 1.f, s = 0.f;
+        if (q < M) {
+          const float apq = Sf[p][q], app = Sf[p][p], aqq = Sf[q][q];
+          // as in the seed pass beyond 32 modes: FP32 rounding keeps tighter thresholds rotating
+          if (apq * apq > 1e-10f * fabsf(app * aqq) && fabsf(apq) > 1e-7f) {
+            const float th = __fdividef(aqq - app, 2.f * apq), h = fmaf(th, th, 1.f);
+            float t = fabsf(th) < 1e18f ? __fdividef(1.f, fabsf(th) + h * rsqrtf(h)) : 0.f;
+            if (th < 0.f) t = -t;
+            c = rsqrtf(fmaf(t, t, 1.f));
+            s = t * c;
+            turned = 1;
+          }
+        }
+        fc[tid] = c;
+        fs[tid] = s;
+        fp[tid] = p;
+        fq[tid] = q;
+      }
+      __syncthreads();
+      if (bk < half) {
+        const float sk = fs[bk], sl = fs[bl], ck = fc[bk], cl = fc[bl];
+        if (sk != 0.f || sl != 0.f) {
+          const int pk = fp[bk], qk = fq[bk], pl = fp[bl], ql = fq[bl];
+          const float b00 = Sf[pk][pl], b01 = Sf[pk][ql], b10 = Sf[qk][pl], b11 = Sf[qk][ql];
+          const float t00 = cl * b00 - sl * b01, t01 = sl * b00 + cl * b01;
+          const float t10 = cl * b10 - sl * b11, t11 = sl * b10 + cl * b11;
+          Sf[pk][pl] = ck * t00 - sk * t10;
+          Sf[pk][ql] = bk == bl ? 0.f : ck * t01 - sk * t11;
+          Sf[qk][pl] = bk == bl ? 0.f : sk * t00 + ck * t10;
+          Sf[qk][ql] = sk * t01 + ck * t11;
+        }
+      }
+      if (vl < half) {
+        const float s = fs[vl];
+        if (s != 0.f) {
+          const int p = fp[vl], q = fq[vl];
+          const float c = fc[vl], vp = Vf[vi][p], vq = Vf[vi][q];
+          Vf[vi][p] = c * vp - s * vq;
+          Vf[vi][q] = s * vp + c * vq;
+        }
+      }
+      __syncthreads();
+    }
+    const bool done = !turned;
+    if (!done && tid == 0) any = 1;
+    __syncthreads();
+    if (done) break;
+  }
+  if (!any) return false;
+  for (int idx = tid; idx < M * M; idx += nt) V[idx / M][idx % M] = (double)Vf[idx / M][idx % M];
+  __syncthreads();
+  md_mm(T, V, V, M, true);   // over the FP32 matrices, which are done with
+  __syncthreads();
+  for (int idx = tid; idx < M * M; idx += nt) {
+    const int i = idx / M, j = idx % M;
+    T[i][j] = (i == j ? 1.0 : 0.0) - T[i][j];
+  }
+  __syncthreads();
+  md_mm(X, T, T, M, false);
+  __syncthreads();
+  for (int idx = tid; idx < M * M; idx += nt) {
+    const int i = idx / M, j = idx % M;
+    T[i][j] = fma(0.375, X[i][j], 0.5 * T[i][j]);
+  }
+  __syncthreads();
+  md_mm(X, V, T, M, false);
+  __syncthreads();
+  for (int idx = tid; idx < M * M; idx += nt) V[idx / M][idx % M] += X[idx / M][idx % M];
+  __syncthreads();
+  md_mm(X, S, V, M, false);
+  __syncthreads();
+  md_mm(T, V, X, M, true);
+  __syncthreads();
+  for (int idx = tid; idx < M * M; idx += nt) {
+    const int i = idx / M, j = idx % M;
+    S[i][j] = 0.5 * (T[i][j] + T[j][i]);
+  }
+  __syncthreads();
+  return true;
 }
 
 // Wp / Wout: the dim's basis from its previous solve (valid when *wM == M) and the
@@ -133,25 +276,13 @@ __global__ void __launch_bounds__(MD_THREADS) md_eig_kernel(const double* __rest
     }
     __syncthreads();
   }
-  // X = L^-1 C_Y into V (thread per column), then S = L^-1 X^T (thread per column)
-  if (tid < M) {
-    const int col = tid;
-    for (int i = 0; i < M; ++i) {
-      double s = S[i][col];
-      for (int j = 0; j < i; ++j) s -= L[i][j] * V[j][col];
-      V[i][col] = s * linv[i];
-    }
-  }
+  // X = L^-1 C_Y into V, then S = L^-1 X^T
+  for (int idx = tid; idx < M * M; idx += nt) V[idx / M][idx % M] = S[idx / M][idx % M];
   __syncthreads();
-  if (tid < M) {
-    const int col = tid;
-    for (int i = 0; i < M; ++i) {
-      double s = V[col][i];
-      for (int j = 0; j < i; ++j) s -= L[i][j] * S[j][col];
-      S[i][col] = s * linv[i];
-    }
-  }
+  md_lsolve(V, L, linv, M);
+  for (int idx = tid; idx < M * M; idx += nt) S[idx / M][idx % M] = V[idx % M][idx / M];
   __syncthreads();
+  md_lsolve(S, L, linv, M);
   for (int idx = tid; idx < M * M; idx += nt) {
     const int i = idx / M, j = idx % M;
     if (i < j) {
@@ -162,6 +293,12 @@ __global__ void __launch_bounds__(MD_THREADS) md_eig_kernel(const double* __rest
     V[i][j] = (i == j) ? 1.0 : 0.0;
   }
   __syncthreads();
+  if (md_seed_rotations(S, V, T, Pw, M)) {
+    // S and V are those of the seed now; the previous basis again
+    for (int idx = tid; idx < M * M; idx += nt)
+      Pw[idx / M][idx % M] = warm ? Wio[idx] : (idx / M == idx % M ? 1.0 : 0.0);
+    __syncthreads();
+  }
   // cyclic Jacobi, round-robin pairing: N = M rounded up to even players, N - 1
   // rounds of N / 2 disjoint pairs per sweep; a pair with the padding player idles
   // (its rotation is the identity; the padding row and column of S are zero)
@@ -173,6 +310,17 @@ __global__ void __launch_bounds__(MD_THREADS) md_eig_kernel(const double* __rest
     }
     __syncthreads();
   }
+  // the thread's block (k <= l) of S, counted along the rows of a triangle (rows k and
+  // half - 1 - k make one row of half + 1), and its entry pair of V: the same in every round
+  int bk = tid / (half + 1), bl = tid % (half + 1);
+  const bool has_block = tid < half * (half + 1) / 2;
+  if (bl <= bk) {
+    bk = half - 1 - bk;
+    bl = half - 1 - bl;
+  } else {
+    --bl;
+  }
+  const int vl = tid / M, vi = tid % M;
   for (int sw = 0; sw < MD_MAX_SWEEPS && M > 1; ++sw) {
     if (tid == 0) rotated = 0;
     __syncthreads();
@@ -183,8 +331,8 @@ __global__ void __launch_bounds__(MD_THREADS) md_eig_kernel(const double* __rest
           a = r;
           b = N - 1;
         } else {
-          a = (r + tid) % (N - 1);
-          b = (r - tid + N - 1) % (N - 1);
+          a = r + tid < N - 1 ? r + tid : r + tid - (N - 1);
+          b = r - tid < 0 ? r - tid + N - 1 : r - tid;
         }
         const int p = min(a, b), q = max(a, b);
         double cs = 1.0, sn = 0.0;
@@ -214,11 +362,9 @@ __global__ void __launch_bounds__(MD_THREADS) md_eig_kernel(const double* __rest
       // S <- J^T S J by 2 x 2 blocks of the round's pairs (k <= l; the lower block is
       // the transpose, the annihilated entry of a diagonal block is set to zero), and
       // V <- V J by row pairs, in one pass: the blocks and the row pairs are disjoint
-      for (int idx = tid; idx < half * half; idx += nt) {
-        const int k = idx / half, l = idx % half;
-        if (k > l) continue;
+      if (has_block && (rs[bk] != 0.0 || rs[bl] != 0.0)) {
+        const int k = bk, l = bl;
         const double sk = rs[k], sl = rs[l];
-        if (sk == 0.0 && sl == 0.0) continue;
         const double ck = rc[k], cl = rc[l];
         const int pk = rp[k], qk = rq[k], pl = rp[l], ql = rq[l];
         // B J_l
@@ -244,15 +390,14 @@ __global__ void __launch_bounds__(MD_THREADS) md_eig_kernel(const double* __rest
           S[ql][qk] = n11;
         }
       }
-      for (int idx = tid; idx < half * M; idx += nt) {
-        const int l = idx / M, i = idx % M;
-        const double sl = rs[l];
+      if (vl < half) {
+        const double sl = rs[vl];
         if (sl != 0.0) {
-          const double cl = rc[l];
-          const int pl = rp[l], ql = rq[l];
-          const double vp = V[i][pl], vq = V[i][ql];
-          V[i][pl] = cl * vp - sl * vq;
-          V[i][ql] = sl * vp + cl * vq;
+          const double cl = rc[vl];
+          const int pl = rp[vl], ql = rq[vl];
+          const double vp = V[vi][pl], vq = V[vi][ql];
+          V[vi][pl] = cl * vp - sl * vq;
+          V[vi][ql] = sl * vp + cl * vq;
         }
       }
       __syncthreads();
