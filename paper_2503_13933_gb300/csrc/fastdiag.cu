@@ -23,6 +23,7 @@
 
 #include <cooperative_groups.h>
 
+#include "small_lu.cuh"
 #include "taps_internal.cuh"
 
 #define FD_THREADS 1024
@@ -555,30 +556,33 @@ __global__ void fd_phi_kernel(const double* __restrict__ L, const double* __rest
 // ---------------------------------------------------------------------------------
 // Per-solve kernels
 // ---------------------------------------------------------------------------------
-// F[i][m] = sum_r q_r[i] c_r[m]
-__global__ void fd_rhs_kernel(const double* __restrict__ q, const double* __restrict__ c, int Rf, int nf,
-                              int M, double* __restrict__ F) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= nf * M) return;
-  int i = idx / M, m = idx % M;
-  double v = 0.0;
-  for (int r = 0; r < Rf; ++r) v += q[(size_t)r * nf + i] * c[(size_t)r * M + m];
-  F[idx] = v;
+// F[i][m] = sum_r q_r[i] c_r[m], one FMA chain per entry.
+__global__ void __launch_bounds__(128) fd_rhs_kernel(const double* __restrict__ q, const double* __restrict__ c,
+                                                     int Rf, int nf, int M, double* __restrict__ F) {
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (long long)nf * M) return;
+  const int i = (int)(idx / M), m = (int)(idx % M);
+  F[idx] = taps_fma_chain<16>(
+      Rf, [&](int r) { return q[(size_t)r * nf + i]; }, [&](int r) { return c[(size_t)r * M + m]; });
+}
+
+int taps_rhs(const double* q, const double* c, int Rf, int n, int M, double* F, cudaStream_t s) {
+  fd_rhs_kernel<<<(unsigned)(((long long)n * M + 127) / 128), 128, 0, s>>>(q, c, Rf, n, M, F);
+  TAPS_CUDA(cudaGetLastError());
+  return TAPS_OK;
 }
 
 // PQ[r][i] = sum_j PhiT[i][j] q[r][j]: the source vectors of dim d in the eigenbasis
 // of its pencil.  The reduced right-hand side of dim d is F = Q c (c from the other
 // dims), so its transform Phi^T F = (Phi^T Q) c needs only this fixed n x Rf matrix.
-__global__ void fd_pq_kernel(const double* __restrict__ PhiT, const double* __restrict__ q, int n,
-                             int Rf, double* __restrict__ PQ) {
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// (Read through Phi, whose neighbouring threads' entries are neighbours.)
+__global__ void __launch_bounds__(128) fd_pq_kernel(const double* __restrict__ Phi, const double* __restrict__ q, int n,
+                                                    int Rf, double* __restrict__ PQ) {
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)n * Rf) return;
   const int r = (int)(idx / n), i = (int)(idx % n);
-  const double* row = PhiT + (size_t)i * n;
   const double* qr = q + (size_t)r * n;
-  double acc = 0.0;
-  for (int j = 0; j < n; ++j) acc += row[j] * qr[j];
-  PQ[idx] = acc;
+  PQ[idx] = taps_fma_chain<16>(n, [&](int j) { return Phi[(size_t)j * n + i]; }, [&](int j) { return qr[j]; });
 }
 
 // Out[i][m] = sum_j Mat[i][j] In[j][m] (Mat n x n row-major, In n x M row-major).
@@ -867,21 +871,10 @@ __global__ void __launch_bounds__(128) fd_small_solve_quad_kernel(const double* 
   if (bad && lane == 0) taps_flag(status, TAPS_DEV_SINGULAR);
 }
 
-// One CTA per node i (M > 32): solve (mu_i C_A + C_B) y = g_i by LU with partial
-// pivoting in shared memory, the right-hand side carried along as column M.  A step's
-// pivot work is a chain of its own (search, reciprocal, multipliers: ~1200 clocks) beside
-// the trailing update's FP64 issue ((M - p)^2 / 2 clocks), so the two overlap: during step
-// p warp 0 updates column p + 1 first, finds its pivot row (largest magnitude, ties to the
-// smaller row; integer compares of the magnitudes' bit patterns), takes the reciprocal
-// (seed plus refinement) and forms the next step's multipliers l_r = T[r][p+1] / pivot with
-// the lanes over the rows, while warps 1 .. update the other columns, one FMA per entry,
-// T[r][c] -= l_r T[p][c], the threads dealt out over the whole trailing block so that no lane
-// idles at row ends.  Rows change places in a table of row offsets, not in memory, and a step
-// has one barrier.  Warp 0 then substitutes back alone, its lanes holding the right-hand
-// side, with the kept reciprocals.  A zero or non-finite pivot is reported as
-// TAPS_DEV_SINGULAR.  Every entry takes the same FMAs in the same order as with two barriers
-// per step and the pivot search between them.  1534 systems of 100 modes: 1.97 -> 1.32 ms
-// (0.85 ms of FP64 issue).
+// One CTA per node i (M > 32): solve (mu_i C_A + C_B) y = g_i by LU with partial pivoting in
+// shared memory (small_lu.cuh).  A zero or non-finite pivot is reported as
+// TAPS_DEV_SINGULAR.  1534 systems of 100 modes: 1.97 ms with the pivot search between two
+// barriers of a step, 1.32 ms now (0.85 ms of FP64 issue).
 #define FS_THREADS 256
 __global__ void __launch_bounds__(FS_THREADS, 2) fd_small_solve_kernel(const double* __restrict__ CA,
                                                                        const double* __restrict__ CB,
@@ -889,126 +882,23 @@ __global__ void __launch_bounds__(FS_THREADS, 2) fd_small_solve_kernel(const dou
                                                                        const double* __restrict__ G, int M,
                                                                        double* __restrict__ Y, int* status) {
   extern __shared__ double T[];   // [M][M+1]: matrix | rhs
-  __shared__ double invd[TAPS_MAX_M];      // reciprocals of the pivots
-  __shared__ double lmul[2][TAPS_MAX_M];   // multipliers of two steps, by logical row
-  __shared__ int rowat[2][TAPS_MAX_M];     // offset of row r in T, for two steps (rows from the step's on)
-  __shared__ int rowfin[TAPS_MAX_M];       // offsets of the pivot rows
+  __shared__ SmallLu sh;
   const int i = blockIdx.x, tid = threadIdx.x;
-  const int lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   const int ld = M + 1;
   const double mi = mu ? mu[i] : 0.0;
   for (int idx = tid; idx < M * M; idx += FS_THREADS) {
     int r = idx / M, c = idx % M;
     T[r * ld + c] = (CA ? mi * CA[idx] : 0.0) + CB[idx];
   }
-  for (int r = tid; r < M; r += FS_THREADS) {
-    T[r * ld + M] = G[(size_t)i * M + r];
-    rowat[0][r] = r * ld;
-  }
-  __syncthreads();
-  // warp 0: the pivot of step p, whose column is final in T; rows in `at` order on entry,
-  // `to` receives the step's order and `l` its multipliers
-  bool bad = false;
-  auto pivot = [&](int p, const int* at, int* to, double* l) {
-    constexpr int S = TAPS_MAX_M / 32;
-    double v[S];
-    long long best = -1;
-    int br = p;
+  for (int r = tid; r < M; r += FS_THREADS) T[r * ld + M] = G[(size_t)i * M + r];
+  double b[TAPS_MAX_M / 32];
+  bool bad;
+  small_lu_solve<FS_THREADS>(T, M, sh, b, bad);
+  if (tid >= 32) return;
 #pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const int r = p + lane + 32 * s;
-      if (r < M) {
-        v[s] = T[at[r] + p];
-        const long long a = __double_as_longlong(fabs(v[s]));
-        if (a > best) { best = a; br = r; }
-      }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int orr = __shfl_xor_sync(0xffffffffu, br, o);
-      if (ob > best || (ob == best && orr < br)) { best = ob; br = orr; }
-    }
-    const double pv = T[at[br] + p];
-    const bool ok = taps_finite_nonzero(pv);
-    const double inv = ok ? taps_rcp(pv) : 0.0;
-    bad |= !ok;
-    if (lane == 0) {
-      invd[p] = inv;
-      rowfin[p] = at[br];
-    }
-    const double v0 = T[at[p] + p];   // the row that takes br's place
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      const int r = p + lane + 32 * s;
-      if (r < M) {
-        to[r] = at[r == p ? br : (r == br ? p : r)];
-        if (r > p) l[r] = (r == br ? v0 : v[s]) * inv;
-      }
-    }
-  };
-  if (warp == 0) pivot(0, rowat[0], rowat[1], lmul[0]);
-  __syncthreads();
-  for (int p = 0; p < M; ++p) {
-    const int* at = rowat[(p + 1) & 1];   // the order of step p
-    const double* l = lmul[p & 1];
-    const double* prow = T + rowfin[p];
-    if (warp == 0) {
-      if (p + 1 < M) {
-        const double pc = prow[p + 1];
-        for (int r = p + 1 + lane; r < M; r += 32) {
-          double* x = T + at[r] + p + 1;
-          *x = fma(-l[r], pc, *x);
-        }
-        __syncwarp();
-        pivot(p + 1, at, rowat[p & 1], lmul[(p + 1) & 1]);
-      }
-    } else {
-      // columns p + 2 .. M of the rows after p, over warps 1 ..
-      const int w = M - 1 - p, rows = M - 1 - p;   // (the right-hand side among the columns)
-      if (w > 0) {
-        const int t = tid - 32, nt = FS_THREADS - 32;
-        int r = t / w, c = t - r * w;
-        const int dr = nt / w, dc = nt - dr * w;
-        while (r < rows) {
-          double* x = T + at[p + 1 + r] + p + 2 + c;
-          *x = fma(-l[p + 1 + r], prow[p + 2 + c], *x);
-          r += dr;
-          c += dc;
-          if (c >= w) {
-            c -= w;
-            ++r;
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-  if (warp != 0) return;
-  // x_r in the lane that holds row r
-  const int* at = rowfin;
-  constexpr int S = TAPS_MAX_M / 32;
-  double b[S];
-#pragma unroll
-  for (int s = 0; s < S; ++s) {
-    const int r = lane + 32 * s;
-    b[s] = r < M ? T[at[r] + M] : 0.0;
-  }
-#pragma unroll
-  for (int sr = S - 1; sr >= 0; --sr) {
-    for (int r = min(M - 1, 32 * sr + 31); r >= 32 * sr; --r) {
-      const double xr = __shfl_sync(0xffffffffu, b[sr], r & 31) * invd[r];   // 0 for a bad pivot
-      if (lane == (r & 31)) b[sr] = xr;
-#pragma unroll
-      for (int s = 0; s <= sr; ++s) {
-        const int k = lane + 32 * s;
-        if (k < r) b[s] = fma(-T[at[k] + r], xr, b[s]);
-      }
-    }
-  }
-#pragma unroll
-  for (int s = 0; s < S; ++s)
-    if (lane + 32 * s < M) Y[(size_t)i * M + lane + 32 * s] = b[s];
-  if (bad && lane == 0) taps_flag(status, TAPS_DEV_SINGULAR);
+  for (int s = 0; s < TAPS_MAX_M / 32; ++s)
+    if (tid + 32 * s < M) Y[(size_t)i * M + tid + 32 * s] = b[s];
+  if (bad && tid == 0) taps_flag(status, TAPS_DEV_SINGULAR);
 }
 
 // ---------------------------------------------------------------------------------
@@ -1281,7 +1171,7 @@ int taps_fd_solve(taps_problem* P, taps_factors* U, int d, int precision) {
                               slotA >= 0 ? (const double*)E->mu : nullptr, (const double*)P->d_pq[d],
                               (const double*)P->d_c, P->Rf, n, M, Y, P->d_status));
   } else {
-    fd_rhs_kernel<<<(nM + 255) / 256, 256, 0, s>>>(P->d_pq[d], P->d_c, P->Rf, n, M, G);
+    TAPS_TRY(taps_rhs(P->d_pq[d], P->d_c, P->Rf, n, M, G, s));
     if (M <= 32)
       fd_small_solve_warp_kernel<<<n, 32, 0, s>>>(CA, CB, slotA >= 0 ? E->mu : nullptr, G, n, M, Y,
                                                   P->d_status, 1);
@@ -1355,7 +1245,7 @@ int taps_fd_prepare_enqueue(taps_problem* P, int solver, int M, std::vector<FdPe
       const long long tot = (long long)n * P->Rf;
       TAPS_TRY(taps_alloc((void**)&P->d_pq[d], sizeof(double) * (size_t)std::max(tot, 1LL)));
       if (tot > 0)
-        fd_pq_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, P->stream>>>(E->PhiT, P->d_q[d], n, P->Rf,
+        fd_pq_kernel<<<(unsigned)((tot + 127) / 128), 128, 0, P->stream>>>(E->Phi, P->d_q[d], n, P->Rf,
                                                                            P->d_pq[d]);
       TAPS_CUDA(cudaGetLastError());
     }

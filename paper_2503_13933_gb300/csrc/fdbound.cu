@@ -13,18 +13,19 @@
 // and the z_b solve the (nb M) x (nb M) capacitance system
 //     z_b' + sum_b beta_b (sum_i phi_b'[i] phi_b[i] T_i^-1) C_b z_b = sum_i phi_b'[i] w_i.
 //
+//   (taps_rhs)         g_i = sum_r (Phi^T q_r)[i] c_r for every node.
 //   fdw_node_kernel    warp per node: LU of T_i without pivoting, w_i and T_i^-1
 //                      (1 + M right-hand sides, lane = row).
 //   fdw_reduce_kernel  the sums over the nodes: Z_b'b = sum_i phi_b' phi_b T_i^-1 and
 //                      the capacitance right-hand side.
-//   fdw_zc_kernel      the capacitance blocks Z_b'b C_b.
-//   fdw_cap_kernel     one CTA: the capacitance system by Gaussian elimination with
+//   fdw_cap_kernel     one CTA: the capacitance blocks Z_b'b C_b and their system by LU with
 //                      partial pivoting, then u_b = C_b z_b.
 //   fdw_final_kernel   y_i; then the node-side transform U = Phi Y (fd_rowgemm_kernel).
 #include <string.h>
 
 #include <algorithm>
 
+#include "small_lu.cuh"
 #include "taps_internal.cuh"
 
 // Forward and backward substitution with the warp's LU factors (lane r holds row r:
@@ -63,9 +64,8 @@ __device__ __forceinline__ void fdw_warp_solve(const double row[33], double invd
 }
 
 __global__ void __launch_bounds__(32) fdw_node_kernel(const double* __restrict__ CA, const double* __restrict__ CB,
-                                                      const double* __restrict__ mu, const double* __restrict__ pq,
-                                                      const double* __restrict__ c, int Rf, int n, int M,
-                                                      double* __restrict__ X, double* __restrict__ w,
+                                                      const double* __restrict__ mu, const double* __restrict__ G,
+                                                      int n, int M, double* __restrict__ X, double* __restrict__ w,
                                                       int* status) {
   const int i = blockIdx.x, lane = threadIdx.x;
   const bool act = lane < M;
@@ -103,11 +103,9 @@ __global__ void __launch_bounds__(32) fdw_node_kernel(const double* __restrict__
   for (int k = 0; k < 32; ++k)
     if (k == lane) diag = row[k];
   const double invd = (act && fabs(diag) > 0.0 && isfinite(diag)) ? taps_rcp(diag) : 0.0;
-  // w_i = T_i^-1 g_i, g_i = sum_r pq[r][i] c_r
+  // w_i = T_i^-1 g_i
   double g[1];
-  g[0] = 0.0;
-  if (act)
-    for (int r = 0; r < Rf; ++r) g[0] = fma(pq[(size_t)r * n + i], c[r * M + lane], g[0]);
+  g[0] = act ? G[(size_t)i * M + lane] : 0.0;
   fdw_warp_solve<1>(row, invd, g, lane, M, 1);
   if (act) w[(size_t)i * M + lane] = g[0];
   // T_i^-1 (row `lane`, all columns)
@@ -127,7 +125,7 @@ __global__ void __launch_bounds__(32) fdw_node_kernel(const double* __restrict__
 
 // Z[b'][b][r][c] = sum_i phi_b'[i] phi_b[i] T_i^-1[r][c];  rr[b'][r] = sum_i phi_b'[i] w_i[r].
 // phi_b[i] = Phi[corner_b][i] (row corner_b of Phi: Phi^T e_b).  X holds T_i^-1.
-__global__ void fdw_reduce_kernel(const double* __restrict__ X, const double* __restrict__ w,
+__global__ void __launch_bounds__(64) fdw_reduce_kernel(const double* __restrict__ X, const double* __restrict__ w,
                                   const double* __restrict__ Phi, int c0, int c1, int n, int M, int nbnd,
                                   double* __restrict__ Z, double* __restrict__ rr) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -136,104 +134,84 @@ __global__ void fdw_reduce_kernel(const double* __restrict__ X, const double* __
     const int cc = idx % M, r = (idx / M) % M, b = (idx / (M * M)) % nbnd, bp = idx / (M * M * nbnd);
     const double* pb = Phi + (size_t)(b == 0 ? c0 : c1) * n;
     const double* pbp = Phi + (size_t)(bp == 0 ? c0 : c1) * n;
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s = fma(pbp[i] * pb[i], X[((size_t)i * M + r) * M + cc], s);
-    Z[idx] = s;
+    Z[idx] = taps_fma_chain<16>(
+        n, [&](int i) { return pbp[i] * pb[i]; }, [&](int i) { return X[((size_t)i * M + r) * M + cc]; });
   } else if (idx < nsc + nbnd * M) {
     const int k = idx - nsc, r = k % M, bp = k / M;
     const double* pbp = Phi + (size_t)(bp == 0 ? c0 : c1) * n;
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s = fma(pbp[i], w[(size_t)i * M + r], s);
-    rr[k] = s;
+    rr[k] = taps_fma_chain<16>(n, [&](int i) { return pbp[i]; }, [&](int i) { return w[(size_t)i * M + r]; });
   }
 }
 
-// SC[b'][b] = Z[b'][b] C_b (M x M products).
-__global__ void fdw_zc_kernel(const double* __restrict__ Z, const double* __restrict__ C0,
-                              const double* __restrict__ C1, int M, int nbnd, double* __restrict__ SC) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= nbnd * nbnd * M * M) return;
-  const int cc = idx % M, r = (idx / M) % M, b = (idx / (M * M)) % nbnd;
-  const double* Cb = b == 0 ? C0 : C1;
-  const double* zr = Z + (size_t)(idx - cc);   // row r of Z[b'][b]
-  double s = 0.0;
-  for (int k = 0; k < M; ++k) s = fma(zr[k], Cb[(size_t)k * M + cc], s);
-  (void)r;
-  SC[idx] = s;
-}
-
-// (I + [beta_b SC[b'][b]]) z = rr, N2 = nbnd M <= 64 unknowns, partial pivoting; beta_b
+// (I + [beta_b Z[b'][b] C_b]) z = rr, N2 = nbnd M <= 64 unknowns, partial pivoting; beta_b
 // is the corner entry of face b's point-mass band.  Writes u_b = C_b z_b and beta for the
 // final kernel.
+// One CTA (small_lu.cuh: the pivot search of a single thread, a row per thread and a single
+// thread's back substitution took 150 us for 40 unknowns).
 #define FDW_MAXN 64
-__global__ void __launch_bounds__(64) fdw_cap_kernel(const double* __restrict__ SC, const double* __restrict__ rr,
+#define FDW_CAP_THREADS 256
+__global__ void __launch_bounds__(FDW_CAP_THREADS) fdw_cap_kernel(const double* __restrict__ Z, const double* __restrict__ rr,
                                                      const double* __restrict__ band0,
                                                      const double* __restrict__ band1, int corner0, int corner1,
                                                      int hb, int M, int nbnd, const double* __restrict__ C0,
                                                      const double* __restrict__ C1, double* __restrict__ z,
                                                      double* __restrict__ beta, int* status) {
-  __shared__ double A[FDW_MAXN][FDW_MAXN + 1];
-  __shared__ double bet[2];
-  __shared__ int piv;
-  const int tid = threadIdx.x, N2 = nbnd * M, nb = 2 * hb + 1;
+  __shared__ double A[FDW_MAXN * (FDW_MAXN + 1)];
+  __shared__ SmallLu sh;
+  __shared__ double bet[2], zs[FDW_MAXN];
+  const int tid = threadIdx.x, N2 = nbnd * M, nb = 2 * hb + 1, ld = N2 + 1;
   if (tid < nbnd) {
     const double* bd = tid == 0 ? band0 : band1;
     const int cr = tid == 0 ? corner0 : corner1;
     bet[tid] = bd[(size_t)cr * nb + hb];
   }
   __syncthreads();
-  for (int idx = tid; idx < N2 * N2; idx += blockDim.x) {
+  // Z into the matrix's place, the products Z[b'][b] C_b in registers, then the matrix
+  for (int idx = tid; idx < N2 * N2; idx += FDW_CAP_THREADS) {
     const int rI = idx / N2, cI = idx % N2;
     const int bp = rI / M, r = rI % M, b = cI / M, cc = cI % M;
-    A[rI][cI] = (rI == cI ? 1.0 : 0.0) + bet[b] * SC[(((size_t)bp * nbnd + b) * M + r) * M + cc];
+    A[rI * ld + cI] = Z[(((size_t)bp * nbnd + b) * M + r) * M + cc];
   }
-  for (int rI = tid; rI < N2; rI += blockDim.x) A[rI][N2] = rr[rI];
-  if (tid < nbnd) beta[tid] = bet[tid];
   __syncthreads();
-  for (int k = 0; k < N2; ++k) {
-    if (tid == 0) {
-      int best = k;
-      double bv = fabs(A[k][k]);
-      for (int rI = k + 1; rI < N2; ++rI)
-        if (fabs(A[rI][k]) > bv) {
-          bv = fabs(A[rI][k]);
-          best = rI;
-        }
-      piv = best;
-      if (!(bv > 0.0) || !isfinite(bv)) taps_flag(status, TAPS_DEV_SINGULAR);
-    }
-    __syncthreads();
-    const int pr = piv;
-    if (pr != k)
-      for (int cI = tid; cI <= N2; cI += blockDim.x) {
-        const double t = A[k][cI];
-        A[k][cI] = A[pr][cI];
-        A[pr][cI] = t;
-      }
-    __syncthreads();
-    const double d = A[k][k];
-    const double id = (fabs(d) > 0.0 && isfinite(d)) ? taps_rcp(d) : 0.0;
-    for (int rI = k + 1 + tid; rI < N2; rI += blockDim.x) {
-      const double l = A[rI][k] * id;
-      for (int cI = k + 1; cI <= N2; ++cI) A[rI][cI] -= l * A[k][cI];
-    }
-    __syncthreads();
+  constexpr int PER = FDW_MAXN * FDW_MAXN / FDW_CAP_THREADS;
+  double v[PER];
+#pragma unroll
+  for (int e = 0; e < PER; ++e) {
+    const int idx = tid + e * FDW_CAP_THREADS;
+    if (idx >= N2 * N2) break;
+    const int rI = idx / N2, cI = idx % N2, b = cI / M, cc = cI % M;
+    const double* Cb = b == 0 ? C0 : C1;
+    const double* zr = A + rI * ld + b * M;
+    double sum = 0.0;
+#pragma unroll 4
+    for (int k = 0; k < M; ++k) sum = fma(zr[k], Cb[(size_t)k * M + cc], sum);
+    v[e] = (rI == cI ? 1.0 : 0.0) + bet[b] * sum;
   }
-  if (tid == 0) {
-    for (int k = N2 - 1; k >= 0; --k) {
-      double s = A[k][N2];
-      for (int cI = k + 1; cI < N2; ++cI) s -= A[k][cI] * A[cI][N2];
-      const double d = A[k][k];
-      A[k][N2] = (fabs(d) > 0.0 && isfinite(d)) ? s * taps_rcp(d) : 0.0;
-    }
+  __syncthreads();
+#pragma unroll
+  for (int e = 0; e < PER; ++e) {
+    const int idx = tid + e * FDW_CAP_THREADS;
+    if (idx >= N2 * N2) break;
+    A[idx / N2 * ld + idx % N2] = v[e];
+  }
+  for (int rI = tid; rI < N2; rI += FDW_CAP_THREADS) A[rI * ld + N2] = rr[rI];
+  if (tid < nbnd) beta[tid] = bet[tid];
+  double x[TAPS_MAX_M / 32];
+  bool bad;
+  small_lu_solve<FDW_CAP_THREADS>(A, N2, sh, x, bad);
+  if (tid < 32) {
+#pragma unroll
+    for (int s = 0; s < FDW_MAXN / 32; ++s)
+      if (tid + 32 * s < N2) zs[tid + 32 * s] = x[s];
+    if (bad && tid == 0) taps_flag(status, TAPS_DEV_SINGULAR);
   }
   __syncthreads();
   // u_b = C_b z_b, stored in z's place (the final kernel needs only u)
-  for (int rI = tid; rI < N2; rI += blockDim.x) {
+  for (int rI = tid; rI < N2; rI += FDW_CAP_THREADS) {
     const int b = rI / M, r = rI % M;
     const double* Cb = b == 0 ? C0 : C1;
     double u = 0.0;
-    for (int k = 0; k < M; ++k) u = fma(Cb[(size_t)r * M + k], A[b * M + k][N2], u);
+    for (int k = 0; k < M; ++k) u = fma(Cb[(size_t)r * M + k], zs[b * M + k], u);
     z[rI] = u;
   }
 }
@@ -293,9 +271,9 @@ int taps_fdw_eligible(const taps_problem* P, int d, int M, int* slotA, int* slot
   return 1;
 }
 
-// T_i^-1 [nf_max][M][M], w [nf_max][M], Z and SC [4][M][M] each, rr, z / u, beta.
+// T_i^-1 [nf_max][M][M], w [nf_max][M], Z [4][M][M], rr, z / u, beta.
 size_t taps_fdw_scratch_doubles(int nf_max, int M) {
-  return (size_t)nf_max * ((size_t)M * M + M) + 8 * (size_t)M * M + 4 * (size_t)M + 8;
+  return (size_t)nf_max * ((size_t)M * M + M) + 4 * (size_t)M * M + 4 * (size_t)M + 8;
 }
 
 // Reduced solve of dim d (coefficients in P->d_C / P->d_c) through the pencil of its
@@ -314,8 +292,7 @@ int taps_fdw_solve(taps_problem* P, taps_factors* U, int d) {
   double* X = P->d_fdw;                        // T_i^-1
   double* w = X + (size_t)P->nf_max * MM;
   double* Z = w + (size_t)P->nf_max * M;
-  double* SC = Z + 4 * MM;
-  double* rr = SC + 4 * MM;
+  double* rr = Z + 4 * MM;
   double* z = rr + 2 * (size_t)M;
   double* beta = z + 2 * (size_t)M;
   double* Y = P->d_Y + (size_t)n * M;
@@ -325,13 +302,14 @@ int taps_fdw_solve(taps_problem* P, taps_factors* U, int d) {
   const double* C0 = P->d_C + (size_t)s0 * MM;
   const double* C1 = s1 >= 0 ? P->d_C + (size_t)s1 * MM : C0;
   int tk = prof_begin(P, TAPS_PROF_FASTDIAG);
-  fdw_node_kernel<<<n, 32, 0, s>>>(P->d_C + (size_t)sa * MM, P->d_C + (size_t)sb * MM, E->mu, P->d_pq[d], P->d_c,
-                                   P->Rf, n, M, X, w, P->d_status);
+  // g_i for every node first: inside the node's one warp, hundreds of source terms' loads were
+  // most of its time
+  TAPS_TRY(taps_rhs(P->d_pq[d], P->d_c, P->Rf, n, M, P->d_Y, s));
+  fdw_node_kernel<<<n, 32, 0, s>>>(P->d_C + (size_t)sa * MM, P->d_C + (size_t)sb * MM, E->mu, P->d_Y, n, M, X, w,
+                                   P->d_status);
   const int nred = nbnd * nbnd * M * M + nbnd * M;
-  fdw_reduce_kernel<<<(nred + 127) / 128, 128, 0, s>>>(X, w, E->Phi, corner0, corner1, n, M, nbnd, Z, rr);
-  const int nzc = nbnd * nbnd * M * M;
-  fdw_zc_kernel<<<(nzc + 127) / 128, 128, 0, s>>>(Z, C0, C1, M, nbnd, SC);
-  fdw_cap_kernel<<<1, 64, 0, s>>>(SC, rr, dm->d_band + (size_t)k0 * bsz, dm->d_band + (size_t)k1 * bsz, corner0,
+  fdw_reduce_kernel<<<(nred + 63) / 64, 64, 0, s>>>(X, w, E->Phi, corner0, corner1, n, M, nbnd, Z, rr);
+  fdw_cap_kernel<<<1, FDW_CAP_THREADS, 0, s>>>(Z, rr, dm->d_band + (size_t)k0 * bsz, dm->d_band + (size_t)k1 * bsz, corner0,
                                   corner1, hb, M, nbnd, C0, C1, z, beta, P->d_status);
   const long long nM = (long long)n * M;
   fdw_final_kernel<<<(unsigned)((nM + 255) / 256), 256, 0, s>>>(X, w, z, beta, E->Phi, corner0, corner1, n, M,

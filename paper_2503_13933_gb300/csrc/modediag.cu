@@ -16,7 +16,7 @@
 //                    Cholesky C_X = L L^T, S = L^-1 C_Y L^-T, cyclic Jacobi
 //                    S = Q diag(lam) Q^T, W = P L^-T Q, and Wc_r = W^T c_r for the
 //                    right-hand side F W = sum_r q_r (W^T c_r)^T.
-//   md_rhs_kernel    every system's right-hand side (F W)_j.
+//   (taps_rhs)       every system's right-hand side (F W)_j = sum_r q_r (W^T c_r)_j.
 //   md_band_kernel   warp j: Gaussian elimination without pivoting of the banded system
 //                    Op_X + lam_j Op_Y (half-bandwidth HB), the lanes sharing a step,
 //                    then back substitution; Z is n_d x M row-major.
@@ -1440,37 +1440,6 @@ __global__ void md_cw_kernel(const double* __restrict__ c, const double* __restr
   cw[idx] = s;
 }
 
-// Fw[i][j] = (F W)[i][j] = sum_r q_r[i] Wc_r[j], one FMA chain per entry; the next sixteen terms
-// are loaded while sixteen are added (a moving source has hundreds).
-__global__ void md_rhs_kernel(const double* __restrict__ q, const double* __restrict__ cw, int Rf, int n, int M,
-                              double* __restrict__ Fw) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)n * M) return;
-  const int j = (int)(idx % M), i = (int)(idx / M);
-  constexpr int T = 16;
-  double a[2][T], b[2][T], v = 0.0;
-  auto load = [&](int r0, double* x, double* y) {
-#pragma unroll
-    for (int t = 0; t < T; ++t) {
-      x[t] = r0 + t < Rf ? q[(size_t)(r0 + t) * n + i] : 0.0;
-      y[t] = r0 + t < Rf ? cw[(size_t)(r0 + t) * M + j] : 0.0;
-    }
-  };
-  auto add = [&](int r0, const double* x, const double* y) {
-#pragma unroll
-    for (int t = 0; t < T; ++t)
-      if (r0 + t < Rf) v = fma(x[t], y[t], v);
-  };
-  load(0, a[0], b[0]);
-  for (int r0 = 0; r0 < Rf; r0 += 2 * T) {
-    load(r0 + T, a[1], b[1]);
-    add(r0, a[0], b[0]);
-    load(r0 + 2 * T, a[0], b[0]);
-    add(r0 + T, a[1], b[1]);
-  }
-  Fw[idx] = v;
-}
-
 // Warp j solves (Op_X + lam_j Op_Y) z_j = (F W)_j by Gaussian elimination without pivoting (no
 // fill outside the band).  An FP64 instruction costs its sub-partition ~64 clocks whatever its
 // active lanes, so the lanes share one system's step (one thread per system: 45 instructions a
@@ -1689,7 +1658,7 @@ template <int HB>
 static cudaError_t md_band_launch(const double* bx, const double* by, const double* lam, const double* q,
                                   const double* cw, int Rf, int n, int M, double* Fw, double* scratch, double* Z,
                                   int* status, cudaStream_t s) {
-  md_rhs_kernel<<<(unsigned)(((long long)n * M + 127) / 128), 128, 0, s>>>(q, cw, Rf, n, M, Fw);
+  if (taps_rhs(q, cw, Rf, n, M, Fw, s) != TAPS_OK) return cudaErrorLaunchFailure;   // (F W)_j
   md_band_kernel<HB><<<M, 32, 0, s>>>(bx, by, lam, Fw, n, M, scratch, Z, status);
   return cudaGetLastError();
 }

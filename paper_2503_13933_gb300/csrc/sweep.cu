@@ -1351,8 +1351,8 @@ __global__ void __launch_bounds__(256) als_residual_all_kernel(ResDims rd, int M
     const int i = idx / M, m = idx % M;
     const int gi = r0 + i;
     if (gi < nf) {
-      double f = 0.0;
-      for (int r = 0; r < Rf; ++r) f += q[(size_t)r * nf + gi] * c[(size_t)r * M + m];
+      const double f = taps_fma_chain<8>(
+          Rf, [&](int r) { return q[(size_t)r * nf + gi]; }, [&](int r) { return c[(size_t)r * M + m]; });
       double a = 0.0;
       for (int o = 0; o < nops; ++o) {
         const double* y = Ys + (o * RR + i) * M;

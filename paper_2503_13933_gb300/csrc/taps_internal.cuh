@@ -258,6 +258,34 @@ __device__ __forceinline__ bool taps_finite_nonzero(double x) {
   return u != 0ull && (u >> 52) != 0x7FFull;
 }
 
+// v + a(0) b(0) + a(1) b(1) + ... as one FMA chain in that order, T terms loaded while T are
+// added: a loop of dependent FMAs over memory otherwise waits for its loads (a moving source
+// has hundreds of terms per entry).
+template <int T, typename A, typename B>
+__device__ __forceinline__ double taps_fma_chain(int count, A a, B b, double v = 0.0) {
+  double x[2][T], y[2][T];
+  auto load = [&](int r0, double (&p)[T], double (&q)[T]) {
+#pragma unroll
+    for (int t = 0; t < T; ++t) {
+      p[t] = r0 + t < count ? a(r0 + t) : 0.0;
+      q[t] = r0 + t < count ? b(r0 + t) : 0.0;
+    }
+  };
+  auto add = [&](int r0, const double (&p)[T], const double (&q)[T]) {
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+      if (r0 + t < count) v = fma(p[t], q[t], v);
+  };
+  load(0, x[0], y[0]);
+  for (int r0 = 0; r0 < count; r0 += 2 * T) {
+    load(r0 + T, x[1], y[1]);
+    add(r0, x[0], y[0]);
+    load(r0 + 2 * T, x[0], y[0]);
+    add(r0 + T, x[1], y[1]);
+  }
+  return v;
+}
+
 // Block-wide sum for blockDim.x <= 1024; `red` holds >= 32 T in shared memory.
 template <typename T>
 __device__ __forceinline__ T block_sum(T v, T* red) {
@@ -437,5 +465,7 @@ int taps_ts_ctas(const taps_problem* P, int hb, int M);
 size_t taps_ts_scratch_doubles(int hb, int M);
 int taps_ts_solve(taps_problem* P, taps_factors* U, int d, int nc);
 int taps_fd_eligible(const taps_problem* P, int d, int* slotA, int* slotB);
+// F[i][m] = sum_r q[r][i] c[r][m] (q [Rf][n], c [Rf][M], F [n][M]).
+int taps_rhs(const double* q, const double* c, int Rf, int n, int M, double* F, cudaStream_t s);
 int taps_fd_solve(taps_problem* P, taps_factors* U, int d, int precision);
 void taps_fd_release(taps_dim* dm);
