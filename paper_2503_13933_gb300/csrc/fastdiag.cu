@@ -38,14 +38,52 @@ __global__ void fd_dense_kernel(const double* __restrict__ bandA, const double* 
   B[idx] = in ? bandB[(size_t)i * nb + k] : 0.0;
 }
 
-// Single-CTA part of the pencil decomposition: on exit B holds the banded Cholesky
-// factor L (lower).  S = L^{-1} A L^{-T} follows in fd_lsolve_kernel (twice) and
-// fd_symmetrize_kernel, column-parallel over many CTAs.
-__global__ void __launch_bounds__(FD_THREADS) fd_setup_kernel(double* B, int n, int hb, int* status) {
+// Banded Cholesky B = L L^T (lower factor in place in the dense B; half-bandwidth hb) and the
+// reciprocals of L's diagonal, by one warp with the band in shared memory: a column is a chain
+// of a square root, a division and an update, and more threads only add barriers to it (1024
+// threads, three block barriers a column: 394 us for 254 nodes).
+__global__ void __launch_bounds__(32) fd_cholesky_kernel(const double* __restrict__ band, double* B, int n, int hb,
+                                                         double* __restrict__ linv, int* status) {
+  extern __shared__ double Lb[];   // [n][hb + 1]: entry (i, i - t) at t
+  const int lane = threadIdx.x, W = hb + 1, nb = 2 * hb + 1;
+  for (int idx = lane; idx < n * W; idx += 32) {
+    const int i = idx / W, t = idx - i * W;
+    Lb[idx] = i - t >= 0 ? band[(size_t)i * nb + hb - t] : 0.0;
+  }
+  __syncwarp();
+  for (int k = 0; k < n; ++k) {
+    double piv = Lb[k * W];
+    if (!(piv > 0.0) || !isfinite(piv)) {
+      if (lane == 0) taps_flag(status, TAPS_DEV_SINGULAR);
+      piv = 1.0;
+    }
+    const double lkk = sqrt(piv);
+    const int w = min(n - 1, k + hb) - k;
+    __syncwarp();
+    if (lane == 0) Lb[k * W] = lkk;
+    if (lane >= 1 && lane <= w) Lb[(k + lane) * W + lane] /= lkk;
+    __syncwarp();
+    for (int idx = lane; idx < w * w; idx += 32) {
+      const int x = 1 + idx / w, y = 1 + idx % w;   // rows k + x >= columns k + y
+      if (y <= x) {
+        double* e = Lb + (k + x) * W + (x - y);
+        *e -= Lb[(k + x) * W + x] * Lb[(k + y) * W + y];
+      }
+    }
+    __syncwarp();
+  }
+  for (int idx = lane; idx < n * W; idx += 32) {
+    const int i = idx / W, t = idx - i * W;
+    if (i - t >= 0) B[(size_t)i * n + i - t] = Lb[idx];
+    if (t == 0) linv[i] = taps_rcp(Lb[idx]);
+  }
+}
+
+// The same for a band that does not fit one CTA's shared memory.
+__global__ void __launch_bounds__(FD_THREADS) fd_cholesky_global_kernel(double* B, int n, int hb,
+                                                                        double* __restrict__ linv, int* status) {
   const int tid = threadIdx.x, nt = blockDim.x;
 #define AT(M_, i, j) M_[(size_t)(i) * n + (j)]
-
-  // ---- 1. banded Cholesky of B (lower factor in place; band half-width hb)
   for (int k = 0; k < n; ++k) {
     if (tid == 0) {
       double piv = AT(B, k, k);
@@ -57,6 +95,7 @@ __global__ void __launch_bounds__(FD_THREADS) fd_setup_kernel(double* B, int n, 
     }
     __syncthreads();
     double lkk = AT(B, k, k);
+    if (tid == 0) linv[k] = taps_rcp(lkk);
     int top = min(n - 1, k + hb);
     for (int i = k + 1 + tid; i <= top; i += nt) AT(B, i, k) /= lkk;
     __syncthreads();
@@ -67,22 +106,51 @@ __global__ void __launch_bounds__(FD_THREADS) fd_setup_kernel(double* B, int n, 
     }
     __syncthreads();
   }
-
 #undef AT
 }
 
 // Out[:, c] = L^{-1} (In[:, c] or, with transposed input, In[c, :]^T) for the banded
-// lower factor L (half-bandwidth hb): one thread per column c, the chain of n
-// substitutions with the diagonal's reciprocal; 32-thread CTAs spread the columns over
-// the SMs (each chain is FP64-latency bound).
-__global__ void __launch_bounds__(32) fd_lsolve_kernel(const double* __restrict__ L, const double* __restrict__ In,
-                                                       int n, int hb, int trans_in, double* __restrict__ Out) {
+// lower factor L (half-bandwidth HB): one thread per column c, the chain of n
+// substitutions with the diagonal's reciprocals; 32-thread CTAs spread the columns over
+// the SMs.  The last HB values stay in registers and the factor's rows are loaded FD_AHEAD
+// rows early, so a step is its HB + 1 FP64 instructions (read back from memory, with a
+// reciprocal per step and column: 248 us for 254 nodes).
+#define FD_AHEAD 4
+template <int HB>
+__global__ void __launch_bounds__(32) fd_lsolve_kernel(const double* __restrict__ L, const double* __restrict__ linv,
+                                                       const double* __restrict__ In, int n, int trans_in,
+                                                       double* __restrict__ Out) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n) return;
-  for (int i = 0; i < n; ++i) {
-    double s = trans_in ? In[(size_t)c * n + i] : In[(size_t)i * n + c];
-    for (int j = max(0, i - hb); j < i; ++j) s -= L[(size_t)i * n + j] * Out[(size_t)j * n + c];
-    Out[(size_t)i * n + c] = s * taps_rcp(L[(size_t)i * n + i]);
+  double x[HB];                                   // values of rows i - HB .. i - 1
+  double l[FD_AHEAD][HB], in[FD_AHEAD], li[FD_AHEAD];
+  auto load = [&](int i, double (&p)[HB], double& q, double& r) {
+    if (i >= n) return;
+#pragma unroll
+    for (int t = 0; t < HB; ++t) p[t] = i - HB + t >= 0 ? L[(size_t)i * n + i - HB + t] : 0.0;
+    q = trans_in ? In[(size_t)c * n + i] : In[(size_t)i * n + c];
+    r = linv[i];
+  };
+#pragma unroll
+  for (int t = 0; t < HB; ++t) x[t] = 0.0;
+#pragma unroll
+  for (int a = 0; a < FD_AHEAD; ++a) load(a, l[a], in[a], li[a]);
+  for (int i0 = 0; i0 < n; i0 += FD_AHEAD) {
+#pragma unroll
+    for (int a = 0; a < FD_AHEAD; ++a) {
+      const int i = i0 + a;
+      if (i >= n) break;
+      double s = in[a];
+#pragma unroll
+      for (int t = 0; t < HB; ++t)
+        if (i - HB + t >= 0) s -= l[a][t] * x[t];
+      s = s * li[a];
+      Out[(size_t)i * n + c] = s;
+#pragma unroll
+      for (int t = 0; t + 1 < HB; ++t) x[t] = x[t + 1];
+      x[HB - 1] = s;
+      load(i + FD_AHEAD, l[a], in[a], li[a]);
+    }
   }
 }
 
@@ -203,13 +271,15 @@ __global__ void __launch_bounds__(TD_THREADS)
 // rows' owners (remote shared-memory loads), forms the reflector, computes p_i for its
 // own rows and stores each p_i into every CTA's copy of p; after a cluster barrier
 // every CTA forms w and updates its own rows; a second barrier ends the step.  S never
-// leaves shared memory.
+// leaves shared memory.  Sums over the column run on the warps that hold entries of it and its
+// scalars (square root, division) on one warp; every warp forming them was two thirds of a
+// step (254 nodes: 3.51 -> 1.73 ms, the same bits: the other warps' summands were zeros).
 template <int NC>
 __global__ void __launch_bounds__(TD_THREADS)
     fd_tridiag_dsmem_kernel(const double* __restrict__ A, double* __restrict__ V, double* __restrict__ beta,
                             double* __restrict__ d, double* __restrict__ e, int n) {
   extern __shared__ double tsm[];   // vs [n] | ps [n] | ws [n] | own rows [nr][n]
-  __shared__ double red[32];
+  __shared__ double red[32], sc[4];
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
@@ -226,18 +296,37 @@ __global__ void __launch_bounds__(TD_THREADS)
   }
   cluster.sync();
   for (int k = 0; k + 2 < n; ++k) {
-    const int len = n - k - 1;
+    const int len = n - k - 1, nact = (len + 31) / 32;   // warps with entries of the column
     // column k below the diagonal, from the owners of its rows
-    double s2 = 0.0;
-    for (int t = tid; t < len; t += TD_THREADS) {
-      const int i = k + 1 + t;
-      const double* owner_rows = cluster.map_shared_rank(rows, i % NC);
-      const double x = owner_rows[(size_t)(i / NC) * n + k];
-      vs[t] = x;
-      s2 += x * x;
+    if (warp < nact) {
+      double s2 = 0.0;
+      for (int t = tid; t < len; t += TD_THREADS) {
+        const int i = k + 1 + t;
+        const double* owner_rows = cluster.map_shared_rank(rows, i % NC);
+        const double x = owner_rows[(size_t)(i / NC) * n + k];
+        vs[t] = x;
+        s2 += x * x;
+      }
+      s2 = warp_sum(s2);
+      if (lane == 0) red[warp] = s2;
     }
-    s2 = block_sum(s2, red);
-    if (s2 == 0.0) {   // the same in every CTA
+    __syncthreads();
+    if (warp == 0) {   // the column's scalars once: 32 warps forming them cost 32 times the issue
+      const double s2 = warp_sum(lane < nact ? red[lane] : 0.0);
+      if (lane == 0) {
+        sc[0] = s2;
+        if (s2 != 0.0) {
+          const double x0 = vs[0];
+          const double al = -copysign(sqrt(s2), x0);
+          const double v0 = x0 - al;
+          sc[1] = al;
+          sc[2] = 2.0 / (s2 - x0 * x0 + v0 * v0);
+          vs[0] = v0;
+        }
+      }
+    }
+    __syncthreads();
+    if (sc[0] == 0.0) {   // the same in every CTA
       if (k % NC == rank && tid == 0) d[k] = rows[(size_t)(k / NC) * n + k];
       if (rank == 0 && tid == 0) {
         beta[k] = 0.0;
@@ -246,13 +335,7 @@ __global__ void __launch_bounds__(TD_THREADS)
       cluster.sync();
       continue;
     }
-    const double x0 = vs[0];
-    const double alpha = -copysign(sqrt(s2), x0);
-    const double v0 = x0 - alpha;
-    const double bk = 2.0 / (s2 - x0 * x0 + v0 * v0);
-    __syncthreads();
-    if (tid == 0) vs[0] = v0;
-    __syncthreads();
+    const double alpha = sc[1], bk = sc[2];
     // p_i for own rows i >= k + 1, pushed into every CTA's ps
     const int l0 = (k + 1 - rank + NC - 1) / NC;   // first own row >= k + 1
     for (int l = l0 + warp; l < nr; l += nwarps) {
@@ -264,11 +347,22 @@ __global__ void __launch_bounds__(TD_THREADS)
       if (lane < NC) cluster.map_shared_rank(ps, lane)[i - k - 1] = acc;
     }
     cluster.sync();
-    double pv = 0.0;
-    for (int t = tid; t < len; t += TD_THREADS) pv += ps[t] * vs[t];
-    pv = block_sum(pv, red);
-    const double Kc = 0.5 * bk * pv;
-    for (int t = tid; t < len; t += TD_THREADS) ws[t] = ps[t] - Kc * vs[t];
+    if (warp < nact) {
+      double pv = 0.0;
+      for (int t = tid; t < len; t += TD_THREADS) pv += ps[t] * vs[t];
+      pv = warp_sum(pv);
+      if (lane == 0) red[warp] = pv;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const double pv = warp_sum(lane < nact ? red[lane] : 0.0);
+      if (lane == 0) sc[3] = 0.5 * bk * pv;
+    }
+    __syncthreads();
+    if (warp < nact) {
+      const double Kc = sc[3];
+      for (int t = tid; t < len; t += TD_THREADS) ws[t] = ps[t] - Kc * vs[t];
+    }
     __syncthreads();
     for (int l = l0 + warp; l < nr; l += nwarps) {
       const int i = rank + NC * l - (k + 1);   // index within the trailing block
@@ -307,24 +401,35 @@ __global__ void __launch_bounds__(TD_THREADS)
 // about 11 rounds, or until rounding stops it shrinking.
 // ---------------------------------------------------------------------------------
 // Number of eigenvalues of T below x: the negative pivots of T - x I,
-// q_i = (d_i - x) - e_{i-1}^2 / q_{i-1}; a pivot smaller than pivmin counts as -pivmin.
-__device__ __forceinline__ int fd_sturm_count(const double* __restrict__ d, const double* __restrict__ e,
-                                              int n, double x, double pivmin) {
+// q_i = (d_i - x) - e_{i-1}^2 / q_{i-1}; a pivot smaller than pivmin counts as -pivmin.  d and
+// e^2 in shared memory; signs and magnitudes by integer compares of the bits (an FP64 compare
+// holds the pipe like an FMA: with the squares 8 of them a step, 5 now).
+__device__ __forceinline__ int fd_sturm_count(const double* d, const double* e2, int n, double x, double pivmin) {
+  const long long pbits = __double_as_longlong(pivmin);
+  int cnt = 0;
   double q = d[0] - x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  int cnt = q < 0.0 ? 1 : 0;
+  auto fix = [&] {
+    const long long mag = __double_as_longlong(q) & 0x7fffffffffffffffll;
+    if (mag < pbits) q = -pivmin;
+    cnt += (__double2hiint(q) < 0 && mag <= 0x7ff0000000000000ll) ? 1 : 0;
+  };
+  fix();
 #pragma unroll 4
   for (int i = 1; i < n; ++i) {
-    const double ei = e[i - 1];
-    q = (d[i] - x) - (ei * ei) * taps_rcp(q);
-    if (fabs(q) < pivmin) q = -pivmin;
-    cnt += q < 0.0 ? 1 : 0;
+    q = (d[i] - x) - e2[i - 1] * taps_rcp(q);
+    fix();
   }
   return cnt;
 }
 
 __global__ void fd_bisect_kernel(const double* __restrict__ d, const double* __restrict__ e, int n,
                                  double* __restrict__ lam) {
+  extern __shared__ double bs[];   // d [n], e^2 [n]
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    bs[i] = d[i];
+    bs[n + i] = e[i] * e[i];
+  }
+  __syncthreads();
   const int k = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (k >= n) return;   // whole warps
@@ -356,7 +461,7 @@ __global__ void fd_bisect_kernel(const double* __restrict__ d, const double* __r
     if (it > 0 && !(w < wprev)) break;   // rounding no longer separates the trial points
     wprev = w;
     const double x = lo + w * (double)(lane + 1) / 33.0;
-    const unsigned above = __ballot_sync(0xffffffffu, fd_sturm_count(d, e, n, x, pivmin) > k);
+    const unsigned above = __ballot_sync(0xffffffffu, fd_sturm_count(bs, bs + n, n, x, pivmin) > k);
     const int j = above ? __ffs(above) - 1 : 32;
     const double nhi = (j < 32) ? lo + w * (double)(j + 1) / 33.0 : hi;
     const double nlo = (j > 0) ? lo + w * (double)j / 33.0 : lo;
@@ -464,6 +569,112 @@ __global__ void fd_invit_kernel(const double* __restrict__ d, const double* __re
 #undef ZC
 }
 
+// The same with T, the factors and the iterate in shared memory: IV_COLS eigenvectors to a CTA
+// of one warp.  The passes are chains over the nodes whose global-memory arrays, written and
+// read back by the same thread, were most of their time (254 nodes: 1055 us).
+#define IV_COLS 8
+static size_t iv_smem(int n) { return sizeof(double) * (2 * (size_t)n + 5 * (size_t)n * IV_COLS) + (size_t)n * IV_COLS; }
+
+__global__ void __launch_bounds__(32) fd_invit_smem_kernel(const double* __restrict__ dg, const double* __restrict__ eg,
+                                                           const double* __restrict__ lam, int n,
+                                                           double* __restrict__ Z) {
+  extern __shared__ double ism[];
+  double* d = ism;
+  double* e = ism + n;
+  double* W = ism + 2 * n;                         // [4][n][IV_COLS]: 1/U0, U1, U2, multiplier
+  double* z = W + 4 * (size_t)n * IV_COLS;         // [n][IV_COLS]
+  unsigned char* swap = reinterpret_cast<unsigned char*>(z + (size_t)n * IV_COLS);
+  const int l = threadIdx.x;
+  for (int i = l; i < n; i += 32) {
+    d[i] = dg[i];
+    e[i] = eg[i];
+  }
+  __syncwarp();
+  const int k0 = blockIdx.x * IV_COLS + l;
+  if (l >= IV_COLS || k0 >= n) return;
+  double tnorm = 0.0;   // Gershgorin bound of ||T||
+  for (int i = 0; i < n; ++i)
+    tnorm = fmax(tnorm, fabs(d[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0) + (i + 1 < n ? fabs(e[i]) : 0.0));
+  if (!(tnorm > 0.0)) tnorm = 1.0;
+  const double ctol = 1e-5 * tnorm;
+  if (k0 > 0 && lam[k0] - lam[k0 - 1] <= ctol) return;   // not the first member of its cluster
+  int k1 = k0;
+  while (k1 + 1 < n && lam[k1 + 1] - lam[k1] <= ctol) ++k1;
+  const double tiny = 2.220446049250313e-16 * tnorm;
+#define WA(a, i) W[((size_t)(a) * n + (i)) * IV_COLS + l]
+#define SW(i) swap[(size_t)(i) * IV_COLS + l]
+#define ZC(i) z[(size_t)(i) * IV_COLS + l]
+  for (int k = k0; k <= k1; ++k) {
+    const double lk = lam[k];
+    double ai = d[0] - lk, bi = n > 1 ? e[0] : 0.0;
+    for (int i = 0; i + 1 < n; ++i) {
+      const double ci = e[i], an = d[i + 1] - lk, bn = (i + 2 < n) ? e[i + 1] : 0.0;
+      if (fabs(ai) >= fabs(ci)) {
+        if (ai == 0.0) ai = tiny;
+        const double m = ci / ai;
+        WA(0, i) = 1.0 / ai;
+        WA(1, i) = bi;
+        WA(2, i) = 0.0;
+        WA(3, i) = m;
+        SW(i) = 0;
+        ai = an - m * bi;
+        bi = bn;
+      } else {
+        const double m = ai / ci;
+        WA(0, i) = 1.0 / ci;
+        WA(1, i) = an;
+        WA(2, i) = bn;
+        WA(3, i) = m;
+        SW(i) = 1;
+        ai = bi - m * an;
+        bi = -m * bn;
+      }
+    }
+    if (ai == 0.0) ai = tiny;
+    WA(0, n - 1) = 1.0 / ai;
+    WA(1, n - 1) = 0.0;   // the last row has no super-diagonals
+    WA(2, n - 1) = 0.0;
+    for (int i = 0; i < n; ++i) ZC(i) = 1.0 + 0.5 * sin(0.7 * i + 1.3 * k);
+    for (int it = 0; it < 3; ++it) {
+      double yi = ZC(0);
+#pragma unroll 4
+      for (int i = 0; i + 1 < n; ++i) {
+        double yn = ZC(i + 1);
+        if (SW(i)) {
+          const double t = yi;
+          yi = yn;
+          yn = t;
+        }
+        ZC(i) = yi;
+        yi = yn - WA(3, i) * yi;
+      }
+      ZC(n - 1) = yi;
+      double z1 = 0.0, z2 = 0.0;
+#pragma unroll 4
+      for (int i = n - 1; i >= 0; --i) {
+        const double zi = (ZC(i) - WA(1, i) * z1 - WA(2, i) * z2) * WA(0, i);
+        ZC(i) = zi;
+        z2 = z1;
+        z1 = zi;
+      }
+      for (int j = k0; j < k; ++j) {   // against the cluster's earlier members
+        double dot = 0.0;
+        for (int i = 0; i < n; ++i) dot += Z[(size_t)i * n + j] * ZC(i);
+        for (int i = 0; i < n; ++i) ZC(i) -= dot * Z[(size_t)i * n + j];
+      }
+      double nrm = 0.0;
+#pragma unroll 4
+      for (int i = 0; i < n; ++i) nrm += ZC(i) * ZC(i);
+      const double inv = (nrm > 0.0) ? 1.0 / sqrt(nrm) : 0.0;
+      for (int i = 0; i < n; ++i) ZC(i) *= inv;
+    }
+    for (int i = 0; i < n; ++i) Z[(size_t)i * n + k] = ZC(i);
+  }
+#undef WA
+#undef SW
+#undef ZC
+}
+
 // ---------------------------------------------------------------------------------
 // Symmetric orthogonalisation of the inverse-iteration vectors, first order:
 // Z <- Z - Z E / 2 with E = Z^T Z - I.  Independently computed eigenvectors are
@@ -511,6 +722,7 @@ __global__ void fd_orth_update_kernel(const double* __restrict__ Z, const double
 // on rows r+1 .. n-1 (v_r in row r of V): warp c takes column c through the reflections
 // from the last to the first, the column held in shared memory.
 // ---------------------------------------------------------------------------------
+#define BT_REGS 16   // reflector entries per lane held in registers (n <= 512)
 __global__ void fd_backtransform_kernel(const double* __restrict__ V, const double* __restrict__ beta, int n,
                                         double* __restrict__ Z) {
   extern __shared__ double zs[];   // [warps per CTA][n]
@@ -520,15 +732,52 @@ __global__ void fd_backtransform_kernel(const double* __restrict__ V, const doub
   double* z = zs + (size_t)wl * n;
   for (int i = lane; i < n; i += 32) z[i] = Z[(size_t)i * n + c];
   __syncwarp();
-  for (int r = n - 3; r >= 0; --r) {
-    const double br = beta[r];
-    if (br == 0.0) continue;
-    const double* v = V + (size_t)r * n;
-    double dot = 0.0;
-    for (int i = r + 1 + lane; i < n; i += 32) dot += v[i] * z[i];
-    dot = warp_sum(dot) * br;
-    for (int i = r + 1 + lane; i < n; i += 32) z[i] -= dot * v[i];
-    __syncwarp();
+  if (n <= 32 * BT_REGS) {
+    // the next reflector is loaded while one is applied
+    double v[BT_REGS], nv[BT_REGS], br = 0.0, nbr = 0.0;
+    auto load = [&](int r) {
+      if (r < 0) return;
+      nbr = beta[r];
+#pragma unroll
+      for (int t = 0; t < BT_REGS; ++t) {
+        const int i = r + 1 + lane + 32 * t;
+        nv[t] = i < n ? V[(size_t)r * n + i] : 0.0;
+      }
+    };
+    load(n - 3);
+    for (int r = n - 3; r >= 0; --r) {
+      br = nbr;
+#pragma unroll
+      for (int t = 0; t < BT_REGS; ++t) v[t] = nv[t];
+      load(r - 1);
+      if (br == 0.0) continue;
+      double dot = 0.0;
+#pragma unroll
+      for (int t = 0; t < BT_REGS; ++t) {
+        const int i = r + 1 + lane + 32 * t;
+        if (r + 1 + 32 * t >= n) break;   // the same for every lane
+        if (i < n) dot += v[t] * z[i];
+      }
+      dot = warp_sum(dot) * br;
+#pragma unroll
+      for (int t = 0; t < BT_REGS; ++t) {
+        const int i = r + 1 + lane + 32 * t;
+        if (r + 1 + 32 * t >= n) break;
+        if (i < n) z[i] -= dot * v[t];
+      }
+      __syncwarp();
+    }
+  } else {
+    for (int r = n - 3; r >= 0; --r) {
+      const double br = beta[r];
+      if (br == 0.0) continue;
+      const double* v = V + (size_t)r * n;
+      double dot = 0.0;
+      for (int i = r + 1 + lane; i < n; i += 32) dot += v[i] * z[i];
+      dot = warp_sum(dot) * br;
+      for (int i = r + 1 + lane; i < n; i += 32) z[i] -= dot * v[i];
+      __syncwarp();
+    }
   }
   for (int i = lane; i < n; i += 32) Z[(size_t)i * n + c] = z[i];
 }
@@ -536,17 +785,43 @@ __global__ void fd_backtransform_kernel(const double* __restrict__ V, const doub
 // Phi = L^{-T} Z (L: the banded Cholesky factor in B, lower, half-width hb), Phi^T, and
 // mu = the eigenvalues; one thread per column.  Without an A (single-operator pencil)
 // Z = I and mu = 0.
-__global__ void fd_phi_kernel(const double* __restrict__ L, const double* __restrict__ Z,
-                              const double* __restrict__ lam, int n, int hb, double* __restrict__ Phi,
-                              double* __restrict__ PhiT, double* __restrict__ mu, int* status) {
+template <int HB>
+__global__ void __launch_bounds__(32) fd_phi_kernel(const double* __restrict__ L, const double* __restrict__ linv,
+                                                    const double* __restrict__ Z, const double* __restrict__ lam, int n,
+                                                    double* __restrict__ Phi, double* __restrict__ PhiT,
+                                                    double* __restrict__ mu, int* status) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n) return;
-  for (int i = n - 1; i >= 0; --i) {
-    double sacc = Z ? Z[(size_t)i * n + c] : (i == c ? 1.0 : 0.0);
-    for (int j = i + 1; j <= min(n - 1, i + hb); ++j) sacc -= L[(size_t)j * n + i] * Phi[(size_t)j * n + c];
-    const double v = sacc * taps_rcp(L[(size_t)i * n + i]);
-    Phi[(size_t)i * n + c] = v;
-    PhiT[(size_t)c * n + i] = v;
+  double x[HB];                                   // values of rows i + 1 .. i + HB
+  double l[FD_AHEAD][HB], in[FD_AHEAD], li[FD_AHEAD];
+  auto load = [&](int i, double (&p)[HB], double& q, double& r) {
+    if (i < 0) return;
+#pragma unroll
+    for (int t = 0; t < HB; ++t) p[t] = i + 1 + t < n ? L[(size_t)(i + 1 + t) * n + i] : 0.0;
+    q = Z ? Z[(size_t)i * n + c] : (i == c ? 1.0 : 0.0);
+    r = linv[i];
+  };
+#pragma unroll
+  for (int t = 0; t < HB; ++t) x[t] = 0.0;
+#pragma unroll
+  for (int a = 0; a < FD_AHEAD; ++a) load(n - 1 - a, l[a], in[a], li[a]);
+  for (int i0 = n - 1; i0 >= 0; i0 -= FD_AHEAD) {
+#pragma unroll
+    for (int a = 0; a < FD_AHEAD; ++a) {
+      const int i = i0 - a;
+      if (i < 0) break;
+      double s = in[a];
+#pragma unroll
+      for (int t = 0; t < HB; ++t)
+        if (i + 1 + t < n) s -= l[a][t] * x[t];
+      s = s * li[a];
+      Phi[(size_t)i * n + c] = s;
+      PhiT[(size_t)c * n + i] = s;
+#pragma unroll
+      for (int t = HB - 1; t > 0; --t) x[t] = x[t - 1];
+      x[0] = s;
+      load(i - FD_AHEAD, l[a], in[a], li[a]);
+    }
   }
   const double m = lam ? lam[c] : 0.0;
   mu[c] = m;
@@ -1019,6 +1294,55 @@ static int td_run(double* A, double* V, double* tmp, double* bt, double* dd, dou
   return TAPS_OK;
 }
 
+// The kernels of the half-bandwidths hb = 2 s + 1, s <= TAPS_MAX_S.
+template <template <int> class K, typename... Args>
+static int fd_by_band(int hb, Args... args) {
+  switch (hb) {
+    case 1: K<1>::launch(args...); break;
+    case 3: K<3>::launch(args...); break;
+    case 5: K<5>::launch(args...); break;
+    case 7: K<7>::launch(args...); break;
+    case 9: K<9>::launch(args...); break;
+    default: return TAPS_ERR_INVALID_ARG;
+  }
+  TAPS_CUDA(cudaGetLastError());
+  return TAPS_OK;
+}
+template <int HB>
+struct LsolveLaunch {
+  static void launch(const double* L, const double* linv, const double* In, int n, int trans_in, double* Out,
+                     cudaStream_t s) {
+    fd_lsolve_kernel<HB><<<(n + 31) / 32, 32, 0, s>>>(L, linv, In, n, trans_in, Out);
+  }
+};
+template <int HB>
+struct PhiLaunch {
+  static void launch(const double* L, const double* linv, const double* Z, const double* lam, int n, double* Phi,
+                     double* PhiT, double* mu, int* status, cudaStream_t s) {
+    fd_phi_kernel<HB><<<(n + 31) / 32, 32, 0, s>>>(L, linv, Z, lam, n, Phi, PhiT, mu, status);
+  }
+};
+static int fd_lsolve(const double* L, const double* linv, const double* In, int n, int hb, int trans_in, double* Out,
+                     cudaStream_t s) {
+  return fd_by_band<LsolveLaunch>(hb, L, linv, In, n, trans_in, Out, s);
+}
+static int fd_phi(const double* L, const double* linv, const double* Z, const double* lam, int n, int hb, double* Phi,
+                  double* PhiT, double* mu, int* status, cudaStream_t s) {
+  return fd_by_band<PhiLaunch>(hb, L, linv, Z, lam, n, Phi, PhiT, mu, status, s);
+}
+static int fd_cholesky(const double* band, double* B, int n, int hb, double* linv, int* status, int maxsm,
+                       cudaStream_t s) {
+  const size_t smem = sizeof(double) * (size_t)n * (hb + 1);
+  if (smem + 1024 <= (size_t)maxsm) {
+    TAPS_TRY(taps_allow_dyn_smem((const void*)fd_cholesky_kernel, maxsm));
+    fd_cholesky_kernel<<<1, 32, smem, s>>>(band, B, n, hb, linv, status);
+  } else {
+    fd_cholesky_global_kernel<<<1, FD_THREADS, 0, s>>>(B, n, hb, linv, status);
+  }
+  TAPS_CUDA(cudaGetLastError());
+  return TAPS_OK;
+}
+
 // Enqueues the decomposition of the pencil (opA, opB) of dm on P's stream without
 // waiting for it: the entry is registered at once (pending, with an event recorded
 // after its last kernel) and the temporaries are returned in *T for fd_finish.  An
@@ -1074,21 +1398,29 @@ static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, FdEntry**
     int tk = prof_begin(P, TAPS_PROF_OTHER);
     fd_dense_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(bandA, bandB, n, dm->hb, A, B);
     if (cudaMemsetAsync(V, 0, sizeof(double) * nn, s) != cudaSuccess) { st = TAPS_ERR_CUDA; break; }
-    // banded Cholesky and S (one CTA), then the tridiagonalisation (one cluster)
-    fd_setup_kernel<<<1, FD_THREADS, 0, s>>>(B, n, dm->hb, P->d_status);
+    // banded Cholesky and S, then the tridiagonalisation (one cluster)
+    double* linv = T->tmp + n;   // the tridiagonalisation uses the first n
+    if ((st = fd_cholesky(bandB, B, n, dm->hb, linv, P->d_status, maxsm_optin, s)) != TAPS_OK) break;
     if (hasA) {
       // S = L^{-1} A L^{-T}: X = L^{-1} A into V, S^T = L^{-1} X^T into W, symmetrised into A
-      fd_lsolve_kernel<<<(n + 31) / 32, 32, 0, s>>>(B, A, n, dm->hb, 0, V);
-      fd_lsolve_kernel<<<(n + 31) / 32, 32, 0, s>>>(B, V, n, dm->hb, 1, W);
+      if ((st = fd_lsolve(B, linv, A, n, dm->hb, 0, V, s)) != TAPS_OK) break;
+      if ((st = fd_lsolve(B, linv, V, n, dm->hb, 1, W, s)) != TAPS_OK) break;
       fd_symmetrize_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(W, n, A);
       if (cudaMemsetAsync(V, 0, sizeof(double) * nn, s) != cudaSuccess) { st = TAPS_ERR_CUDA; break; }
       if ((st = td_run(A, V, T->tmp, T->bt, T->dd, T->ee, n, maxsm_optin, s)) != TAPS_OK) break;
       // eigenvalues (warp each), eigenvectors (thread each), back-transform (warp each),
       // all into A, which the tridiagonalisation no longer needs
       // two warps per CTA: the warps' FP64 chains spread over the SMs' sub-partitions
-      fd_bisect_kernel<<<(unsigned)((32LL * n + 63) / 64), 64, 0, s>>>(T->dd, T->ee, n, lam);
-      // one thread per eigenvector in 32-thread CTAs: the chains spread over the SMs
-      fd_invit_kernel<<<(n + 31) / 32, 32, 0, s>>>(T->dd, T->ee, lam, n, A, W);
+      if ((st = taps_allow_dyn_smem((const void*)fd_bisect_kernel, maxsm_optin)) != TAPS_OK) break;
+      fd_bisect_kernel<<<(unsigned)((32LL * n + 63) / 64), 64, sizeof(double) * 2 * n, s>>>(T->dd, T->ee, n, lam);
+      // eigenvectors in shared memory where IV_COLS of them fit (n <= ~670), else one thread per
+      // eigenvector on global arrays, in 32-thread CTAs: the chains spread over the SMs
+      if (iv_smem(n) + 1024 <= (size_t)maxsm_optin) {
+        if ((st = taps_allow_dyn_smem((const void*)fd_invit_smem_kernel, maxsm_optin)) != TAPS_OK) break;
+        fd_invit_smem_kernel<<<(n + IV_COLS - 1) / IV_COLS, 32, iv_smem(n), s>>>(T->dd, T->ee, lam, n, A);
+      } else {
+        fd_invit_kernel<<<(n + 31) / 32, 32, 0, s>>>(T->dd, T->ee, lam, n, A, W);
+      }
       // symmetric orthogonalisation: E in W, the corrected vectors back into A
       const unsigned gnn = (unsigned)((nn + 255) / 256);
       fd_gram_minus_identity_kernel<<<gnn, 256, 0, s>>>(A, n, W);
@@ -1097,12 +1429,15 @@ static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, FdEntry**
         st = TAPS_ERR_CUDA;
         break;
       }
-      const int wpc = std::max(1, std::min(8, (int)(48 * 1024 / (sizeof(double) * (size_t)n))));
+      // few warps per CTA: one to an SM sub-partition while the columns fit the chip that way
+      const int most = std::max(1, std::min(8, (int)(48 * 1024 / (sizeof(double) * (size_t)n))));
+      const int wpc = std::min(most, std::max(1, (n + P->num_sms - 1) / P->num_sms));
       fd_backtransform_kernel<<<(n + wpc - 1) / wpc, 32 * wpc, sizeof(double) * (size_t)n * wpc, s>>>(
           V, T->bt, n, A);
     }
-    fd_phi_kernel<<<(n + 31) / 32, 32, 0, s>>>(B, hasA ? A : nullptr, hasA ? lam : nullptr, n, dm->hb, E.Phi,
-                                                  E.PhiT, E.mu, P->d_status);
+    if ((st = fd_phi(B, linv, hasA ? A : nullptr, hasA ? lam : nullptr, n, dm->hb, E.Phi, E.PhiT, E.mu, P->d_status,
+                     s)) != TAPS_OK)
+      break;
     prof_end(P, TAPS_PROF_OTHER, tk, (10.0 / 3.0) * (double)nn * n, 8.0 * 4.0 * nn);
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) {
