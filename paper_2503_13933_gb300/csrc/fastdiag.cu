@@ -175,6 +175,7 @@ __global__ void fd_symmetrize_kernel(const double* __restrict__ V, int n, double
 // (row k: entries k+1 .. n-1) and beta their factors.
 // ---------------------------------------------------------------------------------
 #define TD_THREADS 1024
+#define TDS_THREADS 512    // S in distributed shared memory: about a warp per row and CTA
 __device__ __forceinline__ void td_cluster_sync() {
   asm volatile(
       "barrier.cluster.arrive.release.aligned;\n\t"
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(TD_THREADS)
 // scalars (square root, division) on one warp; every warp forming them was two thirds of a
 // step (254 nodes: 3.51 -> 1.73 ms, the same bits: the other warps' summands were zeros).
 template <int NC>
-__global__ void __launch_bounds__(TD_THREADS)
+__global__ void __launch_bounds__(TDS_THREADS)
     fd_tridiag_dsmem_kernel(const double* __restrict__ A, double* __restrict__ V, double* __restrict__ beta,
                             double* __restrict__ d, double* __restrict__ e, int n) {
   extern __shared__ double tsm[];   // vs [n] | ps [n] | ws [n] | own rows [nr][n]
@@ -284,13 +285,13 @@ __global__ void __launch_bounds__(TD_THREADS)
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nwarps = TD_THREADS / 32;
+  const int nwarps = TDS_THREADS / 32;
   double* vs = tsm;
   double* ps = tsm + n;
   double* ws = tsm + 2 * n;
   double* rows = tsm + 3 * n;
   const int nr = (n - rank + NC - 1) / NC;   // rows i = rank + NC * l, l < nr
-  for (long long idx = tid; idx < (long long)nr * n; idx += TD_THREADS) {
+  for (long long idx = tid; idx < (long long)nr * n; idx += TDS_THREADS) {
     const int l = (int)(idx / n), j = (int)(idx % n);
     rows[(size_t)l * n + j] = A[(size_t)(rank + NC * l) * n + j];
   }
@@ -300,7 +301,7 @@ __global__ void __launch_bounds__(TD_THREADS)
     // column k below the diagonal, from the owners of its rows
     if (warp < nact) {
       double s2 = 0.0;
-      for (int t = tid; t < len; t += TD_THREADS) {
+      for (int t = tid; t < len; t += TDS_THREADS) {
         const int i = k + 1 + t;
         const double* owner_rows = cluster.map_shared_rank(rows, i % NC);
         const double x = owner_rows[(size_t)(i / NC) * n + k];
@@ -349,7 +350,7 @@ __global__ void __launch_bounds__(TD_THREADS)
     cluster.sync();
     if (warp < nact) {
       double pv = 0.0;
-      for (int t = tid; t < len; t += TD_THREADS) pv += ps[t] * vs[t];
+      for (int t = tid; t < len; t += TDS_THREADS) pv += ps[t] * vs[t];
       pv = warp_sum(pv);
       if (lane == 0) red[warp] = pv;
     }
@@ -361,7 +362,7 @@ __global__ void __launch_bounds__(TD_THREADS)
     __syncthreads();
     if (warp < nact) {
       const double Kc = sc[3];
-      for (int t = tid; t < len; t += TD_THREADS) ws[t] = ps[t] - Kc * vs[t];
+      for (int t = tid; t < len; t += TDS_THREADS) ws[t] = ps[t] - Kc * vs[t];
     }
     __syncthreads();
     for (int l = l0 + warp; l < nr; l += nwarps) {
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(TD_THREADS)
       for (int t = lane; t < len; t += 32) row[t] -= vi * ws[t] + wi * vs[t];
     }
     if (rank == 0) {
-      for (int t = tid; t < len; t += TD_THREADS) V[(size_t)k * n + k + 1 + t] = vs[t];
+      for (int t = tid; t < len; t += TDS_THREADS) V[(size_t)k * n + k + 1 + t] = vs[t];
       if (tid == 0) {
         beta[k] = bk;
         e[k] = alpha;
@@ -609,26 +610,20 @@ __global__ void __launch_bounds__(32) fd_invit_smem_kernel(const double* __restr
     double ai = d[0] - lk, bi = n > 1 ? e[0] : 0.0;
     for (int i = 0; i + 1 < n; ++i) {
       const double ci = e[i], an = d[i + 1] - lk, bn = (i + 2 < n) ? e[i + 1] : 0.0;
-      if (fabs(ai) >= fabs(ci)) {
-        if (ai == 0.0) ai = tiny;
-        const double m = ci / ai;
-        WA(0, i) = 1.0 / ai;
-        WA(1, i) = bi;
-        WA(2, i) = 0.0;
-        WA(3, i) = m;
-        SW(i) = 0;
-        ai = an - m * bi;
-        bi = bn;
-      } else {
-        const double m = ai / ci;
-        WA(0, i) = 1.0 / ci;
-        WA(1, i) = an;
-        WA(2, i) = bn;
-        WA(3, i) = m;
-        SW(i) = 1;
-        ai = bi - m * an;
-        bi = -m * bn;
-      }
+      // both sides of the pivoting in one: its two divisions (a dozen FP64 instructions each)
+      // are not issued for either side
+      const bool keep = fabs(ai) >= fabs(ci);
+      if (keep && ai == 0.0) ai = tiny;
+      const double den = keep ? ai : ci, num = keep ? ci : ai;
+      const double m = num / den;
+      WA(0, i) = 1.0 / den;
+      WA(1, i) = keep ? bi : an;
+      WA(2, i) = keep ? 0.0 : bn;
+      WA(3, i) = m;
+      SW(i) = keep ? 0 : 1;
+      const double upper = keep ? bi : an;
+      ai = (keep ? an : bi) - m * upper;
+      bi = keep ? bn : -m * bn;
     }
     if (ai == 0.0) ai = tiny;
     WA(0, n - 1) = 1.0 / ai;
@@ -1221,7 +1216,7 @@ static void fd_pending_free(FdPending& T) {
 // cluster of the kernel (non-portable size), else the portable 8.  Both variants do the
 // same arithmetic per row and per reduction, so the result does not depend on it.
 template <int NC>
-static bool td_cluster_ok(const void* fn, size_t smem) {
+static bool td_cluster_ok(const void* fn, size_t smem, int threads) {
   if (NC > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
     return false;
@@ -1235,7 +1230,7 @@ static bool td_cluster_ok(const void* fn, size_t smem) {
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(NC);
-  cfg.blockDim = dim3(TD_THREADS);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1253,10 +1248,10 @@ static bool td_cluster_ok(const void* fn, size_t smem) {
 }
 
 template <int NC, typename... Args>
-static cudaError_t td_launch(void (*fn)(Args...), size_t smem, cudaStream_t s, Args... args) {
+static cudaError_t td_launch(void (*fn)(Args...), int threads, size_t smem, cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(NC);
-  cfg.blockDim = dim3(TD_THREADS);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
@@ -1277,15 +1272,15 @@ static int td_run(double* A, double* V, double* tmp, double* bt, double* dd, dou
   const size_t dsm8 = sizeof(double) * ((size_t)((n + 7) / 8) * n + 3 * (size_t)n);
   const size_t gsm = sizeof(double) * 3 * (size_t)n;
   cudaError_t ce;
-  if (dsm16 + 1024 <= (size_t)maxsm && td_cluster_ok<16>((const void*)fd_tridiag_dsmem_kernel<16>, dsm16)) {
-    ce = td_launch<16>(fd_tridiag_dsmem_kernel<16>, dsm16, s, (const double*)A, V, bt, dd, ee, n);
-  } else if (dsm8 + 1024 <= (size_t)maxsm && td_cluster_ok<8>((const void*)fd_tridiag_dsmem_kernel<8>, dsm8)) {
-    ce = td_launch<8>(fd_tridiag_dsmem_kernel<8>, dsm8, s, (const double*)A, V, bt, dd, ee, n);
-  } else if (td_cluster_ok<16>((const void*)fd_tridiag_kernel<16>, gsm)) {
-    ce = td_launch<16>(fd_tridiag_kernel<16>, gsm, s, A, V, tmp, bt, dd, ee, n);
+  if (dsm16 + 1024 <= (size_t)maxsm && td_cluster_ok<16>((const void*)fd_tridiag_dsmem_kernel<16>, dsm16, TDS_THREADS)) {
+    ce = td_launch<16>(fd_tridiag_dsmem_kernel<16>, TDS_THREADS, dsm16, s, (const double*)A, V, bt, dd, ee, n);
+  } else if (dsm8 + 1024 <= (size_t)maxsm && td_cluster_ok<8>((const void*)fd_tridiag_dsmem_kernel<8>, dsm8, TDS_THREADS)) {
+    ce = td_launch<8>(fd_tridiag_dsmem_kernel<8>, TDS_THREADS, dsm8, s, (const double*)A, V, bt, dd, ee, n);
+  } else if (td_cluster_ok<16>((const void*)fd_tridiag_kernel<16>, gsm, TD_THREADS)) {
+    ce = td_launch<16>(fd_tridiag_kernel<16>, TD_THREADS, gsm, s, A, V, tmp, bt, dd, ee, n);
   } else {
-    if (!td_cluster_ok<8>((const void*)fd_tridiag_kernel<8>, gsm)) return TAPS_ERR_CUDA;
-    ce = td_launch<8>(fd_tridiag_kernel<8>, gsm, s, A, V, tmp, bt, dd, ee, n);
+    if (!td_cluster_ok<8>((const void*)fd_tridiag_kernel<8>, gsm, TD_THREADS)) return TAPS_ERR_CUDA;
+    ce = td_launch<8>(fd_tridiag_kernel<8>, TD_THREADS, gsm, s, A, V, tmp, bt, dd, ee, n);
   }
   if (ce != cudaSuccess) {
     taps_note_cuda_error(ce, "tridiagonalisation launch", __FILE__, __LINE__);
