@@ -14,7 +14,7 @@
 //     z_b' + sum_b beta_b (sum_i phi_b'[i] phi_b[i] T_i^-1) C_b z_b = sum_i phi_b'[i] w_i.
 //
 //   (taps_rhs)         g_i = sum_r (Phi^T q_r)[i] c_r for every node.
-//   fdw_node_kernel    warp per node: LU of T_i without pivoting, w_i and T_i^-1
+//   fdw_node_kernel    four warps per node: LU of T_i without pivoting, w_i and T_i^-1
 //                      (1 + M right-hand sides, lane = row).
 //   fdw_reduce_kernel  the sums over the nodes: Z_b'b = sum_i phi_b' phi_b T_i^-1 and
 //                      the capacitance right-hand side.
@@ -28,119 +28,160 @@
 #include "small_lu.cuh"
 #include "taps_internal.cuh"
 
-// Forward and backward substitution with the warp's LU factors (lane r holds row r:
-// unit-lower multipliers left of the diagonal, U on and right of it) for NC
-// right-hand-side columns held as rhs[c] in lane r.  invd is 1 / U[r][r] in lane r.
-template <int NC>
-__device__ __forceinline__ void fdw_warp_solve(const double row[33], double invd, double rhs[NC], int lane,
-                                               int M, int ncol) {
-#pragma unroll
-  for (int p = 0; p < 32; ++p) {
-    if (p < M) {
-      const double l = row[p];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        if (c < ncol) {
-          const double v = __shfl_sync(0xffffffffu, rhs[c], p);
-          if (lane > p && lane < M) rhs[c] -= l * v;
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int p = 31; p >= 0; --p) {
-    if (p < M) {
-      const double u = row[p];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        if (c < ncol) {
-          if (lane == p) rhs[c] *= invd;
-          const double v = __shfl_sync(0xffffffffu, rhs[c], p);
-          if (lane < p) rhs[c] -= u * v;
-        }
-      }
-    }
-  }
-}
-
-__global__ void __launch_bounds__(32) fdw_node_kernel(const double* __restrict__ CA, const double* __restrict__ CB,
-                                                      const double* __restrict__ mu, const double* __restrict__ G,
-                                                      int n, int M, double* __restrict__ X, double* __restrict__ w,
-                                                      int* status) {
-  const int i = blockIdx.x, lane = threadIdx.x;
+// One CTA of four warps per node (M <= 32): T_i = mu_i C_A + C_B factored as L U without
+// pivoting (the symmetric part of T_i is positive definite), then w_i = T_i^-1 g_i and T_i^-1.
+// A warp-wide FP64 instruction holds its SM sub-partition ~64 cycles whatever lanes it uses, so
+// the issue of the M^3-sized work is the bound and it is spread over the four sub-partitions:
+// role w holds the columns c = w, w + 4, ... (lane = row), of T_i first and of the identity
+// after, and the role with the fewest columns takes g_i.  The multipliers and U go to shared
+// memory column by column.  Columns of L^-1 start at their own row; a backward step's M / 4
+// products with the pivot's reciprocal are one multiplication across lanes.  CTAs num_sms apart,
+// which land on one SM, put the same role on different sub-partitions.  255 nodes of 20 modes:
+// 125 us with one warp per node, 36 us now.
+__global__ void __launch_bounds__(128) fdw_node_kernel(const double* __restrict__ CA, const double* __restrict__ CB,
+                                                       const double* __restrict__ mu, const double* __restrict__ G,
+                                                       int n, int M, int num_sms, double* __restrict__ X,
+                                                       double* __restrict__ w, int* status) {
+  __shared__ double LU[32][33];   // [column][row]: multipliers below the diagonal, U on and above it
+  __shared__ double invd[32];
+  const int i = blockIdx.x, lane = threadIdx.x & 31;
+  const int role = ((threadIdx.x >> 5) + 2 * (i / num_sms)) & 3;
   const bool act = lane < M;
   const double mi = mu[i];
-  double row[33];
+  double v[8];
 #pragma unroll
-  for (int k = 0; k < 33; ++k) row[k] = 0.0;
-  if (act) {
-#pragma unroll
-    for (int k = 0; k < 32; ++k)
-      if (k < M) row[k] = fma(mi, CA[lane * M + k], CB[lane * M + k]);
+  for (int k = 0; k < 8; ++k) {
+    const int c = 4 * k + role;
+    v[k] = (act && c < M) ? fma(mi, CA[lane * M + c], CB[lane * M + c]) : 0.0;
   }
-  // LU without pivoting: the symmetric part of T_i is positive definite
+  double g = (role == (M & 3) && act) ? G[(size_t)i * M + lane] : 0.0;
   bool bad = false;
+  // the multipliers of a step and the pivot's reciprocal (0 for a zero or non-finite pivot)
+  auto publish = [&](int q, double col, double piv) {
+    const bool ok = taps_finite_nonzero(piv);
+    bad |= !ok;
+    const double ip = ok ? taps_rcp(piv) : 0.0;
+    LU[q][lane] = (lane > q && act) ? col * ip : 0.0;
+    if (lane == 0) invd[q] = ip;
+  };
+  if (role == 0) publish(0, v[0], __shfl_sync(0xffffffffu, v[0], 0));
+  __syncthreads();
 #pragma unroll
   for (int p = 0; p < 32; ++p) {
     if (p < M) {
-      const double piv = __shfl_sync(0xffffffffu, row[p], p);
-      bad |= !(fabs(piv) > 0.0) || !isfinite(piv);
-      const double ip = (fabs(piv) > 0.0 && isfinite(piv)) ? taps_rcp(piv) : 0.0;
-      const double l = (lane > p && act) ? row[p] * ip : 0.0;
-#pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        if (k > p && k < M) {
-          const double pk = __shfl_sync(0xffffffffu, row[k], p);
-          row[k] -= l * pk;
-        }
+      const double l = LU[p][lane];
+      const int q = p + 1;   // next pivot column, owned by role q & 3 in slot q >> 2
+      const bool owner = q < M && role == (q & 3);
+      if (owner) {
+        v[(q >> 2) & 7] -= l * __shfl_sync(0xffffffffu, v[(q >> 2) & 7], p);
+        publish(q, v[(q >> 2) & 7], __shfl_sync(0xffffffffu, v[(q >> 2) & 7], q & 31));
       }
-      if (lane > p && act) row[p] = l;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {   // this role's columns c > p
+        const int c = 4 * k + role;
+        if (4 * k + 3 <= p || c <= p || c >= M || (owner && c == q)) continue;
+        v[k] -= l * __shfl_sync(0xffffffffu, v[k], p);
+      }
+      __syncthreads();
     }
   }
   if (bad && lane == 0) taps_flag(status, TAPS_DEV_SINGULAR);
-  double diag = 1.0;   // U[lane][lane], selected with compile-time register indices
 #pragma unroll
-  for (int k = 0; k < 32; ++k)
-    if (k == lane) diag = row[k];
-  const double invd = (act && fabs(diag) > 0.0 && isfinite(diag)) ? taps_rcp(diag) : 0.0;
-  // w_i = T_i^-1 g_i
-  double g[1];
-  g[0] = act ? G[(size_t)i * M + lane] : 0.0;
-  fdw_warp_solve<1>(row, invd, g, lane, M, 1);
-  if (act) w[(size_t)i * M + lane] = g[0];
-  // T_i^-1 (row `lane`, all columns)
-  {
-    double rhs[32];
+  for (int k = 0; k < 8; ++k) {
+    const int c = 4 * k + role;
+    if (c < M && lane <= c) LU[c][lane] = v[k];
+  }
+  __syncthreads();
+  // columns of the identity (and g): forward from the column's own row, then backward
 #pragma unroll
-    for (int k = 0; k < 32; ++k) rhs[k] = (act && k == lane) ? 1.0 : 0.0;
-    fdw_warp_solve<32>(row, invd, rhs, lane, M, M);
-    if (act) {
-      double* out = X + ((size_t)i * M + lane) * M;
+  for (int k = 0; k < 8; ++k) v[k] = (act && lane == 4 * k + role) ? 1.0 : 0.0;
+  const bool has_g = role == (M & 3);
+  for (int p = 0; p < M; ++p) {
+    const double l = LU[p][lane];
+    if (has_g) {
+      const double t = __shfl_sync(0xffffffffu, g, p);
+      if (lane > p) g -= l * t;
+    }
 #pragma unroll
-      for (int k = 0; k < 32; ++k)
-        if (k < M) out[k] = rhs[k];
+    for (int k = 0; k < 8; ++k) {
+      const int c = 4 * k + role;
+      if (c > p || c >= M) continue;
+      const double t = __shfl_sync(0xffffffffu, v[k], p);
+      if (lane > p) v[k] -= l * t;
     }
   }
+  for (int p = M - 1; p >= 0; --p) {
+    const double u = LU[p][lane];
+    double xp = has_g ? __shfl_sync(0xffffffffu, g, p) : 0.0;   // row p of slot k in lane k, of g in lane 8
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (4 * k + role >= M) continue;
+      const double t = __shfl_sync(0xffffffffu, v[k], p);
+      if (lane == k) xp = t;
+    }
+    xp *= invd[p];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (4 * k + role >= M) continue;
+      const double t = __shfl_sync(0xffffffffu, xp, k);
+      if (lane == p) v[k] = t;
+      if (lane < p) v[k] -= u * t;
+    }
+    if (has_g) {
+      const double t = __shfl_sync(0xffffffffu, xp, 8);
+      if (lane == p) g = t;
+      if (lane < p) g -= u * t;
+    }
+  }
+  if (has_g && act) w[(size_t)i * M + lane] = g;
+  // T_i^-1 row by row through shared memory (whole-sector stores)
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (4 * k + role < M) LU[4 * k + role][lane] = v[k];
+  __syncthreads();
+  for (int idx = threadIdx.x; idx < M * M; idx += 128) X[(size_t)i * M * M + idx] = LU[idx % M][idx / M];
 }
 
 // Z[b'][b][r][c] = sum_i phi_b'[i] phi_b[i] T_i^-1[r][c];  rr[b'][r] = sum_i phi_b'[i] w_i[r].
 // phi_b[i] = Phi[corner_b][i] (row corner_b of Phi: Phi^T e_b).  X holds T_i^-1.
-__global__ void __launch_bounds__(64) fdw_reduce_kernel(const double* __restrict__ X, const double* __restrict__ w,
-                                  const double* __restrict__ Phi, int c0, int c1, int n, int M, int nbnd,
-                                  double* __restrict__ Z, double* __restrict__ rr) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  const int nsc = nbnd * nbnd * M * M;
-  if (idx < nsc) {
-    const int cc = idx % M, r = (idx / M) % M, b = (idx / (M * M)) % nbnd, bp = idx / (M * M * nbnd);
-    const double* pb = Phi + (size_t)(b == 0 ? c0 : c1) * n;
-    const double* pbp = Phi + (size_t)(bp == 0 ? c0 : c1) * n;
-    Z[idx] = taps_fma_chain<16>(
-        n, [&](int i) { return pbp[i] * pb[i]; }, [&](int i) { return X[((size_t)i * M + r) * M + cc]; });
-  } else if (idx < nsc + nbnd * M) {
-    const int k = idx - nsc, r = k % M, bp = k / M;
-    const double* pbp = Phi + (size_t)(bp == 0 ? c0 : c1) * n;
-    rr[k] = taps_fma_chain<16>(n, [&](int i) { return pbp[i]; }, [&](int i) { return w[(size_t)i * M + r]; });
+// blockIdx.y = the pair (b', b), b' <= b (the weights of (b, b') are the same), then the rows
+// of rr; one warp adds 32 entries over the nodes in order, the products of phi formed once per
+// CTA in shared memory.  The chain of n FMAs is the bound: 255 nodes of 20 modes, two faces,
+// 34 us with the products in every thread and all four pairs, 23 us now.
+#define FDW_RED_NODES 512
+__global__ void __launch_bounds__(32) fdw_reduce_kernel(const double* __restrict__ X, const double* __restrict__ w,
+                                                        const double* __restrict__ Phi, int c0, int c1, int n, int M,
+                                                        int nbnd, double* __restrict__ Z, double* __restrict__ rr) {
+  __shared__ double ph[FDW_RED_NODES];
+  const int e = blockIdx.x * 32 + threadIdx.x, MM = M * M;
+  const int npair = nbnd == 2 ? 3 : 1;
+  const bool pair = (int)blockIdx.y < npair;
+  const int q = pair ? blockIdx.y : blockIdx.y - npair;
+  const int bp = pair ? q >> 1 : q, b = pair ? (q + 1) >> 1 : q;   // (0,0), (0,1), (1,1)
+  const int count = pair ? MM : M;
+  if ((int)blockIdx.x * 32 >= count) return;
+  const double* pb = Phi + (size_t)(b == 0 ? c0 : c1) * n;
+  const double* pbp = Phi + (size_t)(bp == 0 ? c0 : c1) * n;
+  const double* src = pair ? X : w;
+  const int ec = min(e, count - 1);
+  double v = 0.0;
+  for (int i0 = 0; i0 < n; i0 += FDW_RED_NODES) {
+    const int len = min(FDW_RED_NODES, n - i0);
+    __syncwarp();
+    for (int i = threadIdx.x; i < len; i += 32) ph[i] = pair ? pbp[i0 + i] * pb[i0 + i] : pbp[i0 + i];
+    __syncwarp();
+    const double* xs = src + (size_t)i0 * count + ec;
+    v = taps_fma_chain<16>(
+        len, [&](int i) { return ph[i]; }, [&](int i) { return xs[(size_t)i * count]; }, v);
   }
+  if (e >= count) return;
+  if (!pair) {
+    rr[bp * M + e] = v;
+    return;
+  }
+  Z[(size_t)(bp * nbnd + b) * MM + e] = v;
+  if (b != bp) Z[(size_t)(b * nbnd + bp) * MM + e] = v;
 }
 
 // (I + [beta_b Z[b'][b] C_b]) z = rr, N2 = nbnd M <= 64 unknowns, partial pivoting; beta_b
@@ -305,10 +346,10 @@ int taps_fdw_solve(taps_problem* P, taps_factors* U, int d) {
   // g_i for every node first: inside the node's one warp, hundreds of source terms' loads were
   // most of its time
   TAPS_TRY(taps_rhs(P->d_pq[d], P->d_c, P->Rf, n, M, P->d_Y, s));
-  fdw_node_kernel<<<n, 32, 0, s>>>(P->d_C + (size_t)sa * MM, P->d_C + (size_t)sb * MM, E->mu, P->d_Y, n, M, X, w,
-                                   P->d_status);
-  const int nred = nbnd * nbnd * M * M + nbnd * M;
-  fdw_reduce_kernel<<<(nred + 63) / 64, 64, 0, s>>>(X, w, E->Phi, corner0, corner1, n, M, nbnd, Z, rr);
+  fdw_node_kernel<<<n, 128, 0, s>>>(P->d_C + (size_t)sa * MM, P->d_C + (size_t)sb * MM, E->mu, P->d_Y, n, M,
+                                    P->num_sms, X, w, P->d_status);
+  fdw_reduce_kernel<<<dim3((M * M + 31) / 32, nbnd == 2 ? 5 : 2), 32, 0, s>>>(X, w, E->Phi, corner0, corner1, n, M,
+                                                                              nbnd, Z, rr);
   fdw_cap_kernel<<<1, FDW_CAP_THREADS, 0, s>>>(Z, rr, dm->d_band + (size_t)k0 * bsz, dm->d_band + (size_t)k1 * bsz, corner0,
                                   corner1, hb, M, nbnd, C0, C1, z, beta, P->d_status);
   const long long nM = (long long)n * M;
