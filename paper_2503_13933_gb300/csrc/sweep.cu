@@ -22,22 +22,20 @@
 // pipe ~64 cycles on this GPU, so the exact multiplications by 1 of unused dim slots
 // and an add per possible operator slot were most of the work).  Each operator slot's
 // sum takes its terms in increasing order.
-// More distinct operators than TAPS_NUM_OPS (weighted operators): one slot at a time,
-// the terms in the same order, so each slot's sum is the one the register version forms.
-__device__ __forceinline__ void coeff_C_slots(const TermTable& tt, const GramPtrs& gp, int d, int M, int idx,
-                                           double* C) {
+// More distinct operators than TAPS_NUM_OPS (weighted operators): slot o of entry idx, the
+// terms in the same order, so each slot's sum is the one the other version forms.
+__device__ __forceinline__ void coeff_C_slot(const TermTable& tt, const GramPtrs& gp, int d, int M, int o, int idx,
+                                             double* C) {
   const int MM = M * M;
-  for (int o = 0; o < tt.nops[d]; ++o) {
-    double acc = 0.0;
-    for (int t = 0; t < tt.R; ++t) {
-      if (tt.oi[t][d] != o) continue;
-      double prod = tt.alpha[t];
-      for (int e = 0; e < tt.D; ++e)
-        if (e != d) prod *= __ldcg(gp.gram[e] + (size_t)tt.oi[t][e] * MM + idx);
-      acc += prod;
-    }
-    C[(size_t)o * MM + idx] = acc;
+  double acc = 0.0;
+  for (int t = 0; t < tt.R; ++t) {
+    if (tt.oi[t][d] != o) continue;
+    double prod = tt.alpha[t];
+    for (int e = 0; e < tt.D; ++e)
+      if (e != d) prod *= __ldcg(gp.gram[e] + (size_t)tt.oi[t][e] * MM + idx);
+    acc += prod;
   }
+  C[(size_t)o * MM + idx] = acc;
 }
 
 __device__ __forceinline__ void coeff_C(const TermTable& tt, const GramPtrs& gp, int d, int M, int idx,
@@ -95,11 +93,17 @@ __global__ void coeff_all_kernel(TermTable tt, GramPtrs gp, int M, double* Call,
 }
 
 // The same with more distinct operators than TAPS_NUM_OPS in some dim (weighted
-// operators): coefficient arrays with slot stride tt.cs.
-__device__ __forceinline__ void coeff_entry_slots(const TermTable& tt, const GramPtrs& gp, int d, int M, int idx,
+// operators): coefficient arrays with slot stride tt.cs, and a thread per entry of every
+// operator -- a few modes have few entries, and a thread that went through the operators of
+// its entry one after another took 43 us for 12 of them and 6 modes (8 us now).
+__device__ __forceinline__ void coeff_entry_slots(const TermTable& tt, const GramPtrs& gp, int d, int M, int e,
                                                   double* C, double* c) {
-  if (idx < M * M) coeff_C_slots(tt, gp, d, M, idx, C);
-  if (idx < tt.Rf * M) coeff_c(tt, gp, d, M, idx / M, idx % M, c);   // one thread per (r, m)
+  const int MM = M * M, nC = tt.nops[d] * MM;
+  if (e < nC) coeff_C_slot(tt, gp, d, M, e / MM, e % MM, C);
+  else if (e - nC < tt.Rf * M) coeff_c(tt, gp, d, M, (e - nC) / M, (e - nC) % M, c);
+}
+static unsigned coeff_slots_blocks(const taps_problem* P, int nops, int M) {
+  return (unsigned)((nops * M * M + P->Rf * M + 127) / 128);
 }
 
 __global__ void coeff_slots_kernel(TermTable tt, GramPtrs gp, int d, int M, double* C, double* c) {
@@ -139,14 +143,14 @@ __device__ __forceinline__ void gram_partial_body(int chunk, int tile, int nchun
                                                   double* __restrict__ partial, int stride, unsigned* ticket,
                                                   double* gram, double* h, const TermTable& tt,
                                                   const GramPtrs& gp, int cd, double* C, double* c, int gmt,
-                                                  int tail) {
+                                                  int tail, int og) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int is_last;
   const int nb = 2 * hb + 1;
   const int rows_h = GR + 2 * hb;
   T* Us = reinterpret_cast<T*>(smem_raw);  // [rows_h][M]
-  T* Ys = Us + rows_h * M;                 // [GR][M]
-  T* Bs = Ys + GR * M;                     // [nops][GR][nb] the chunk's band rows
+  T* Ys = Us + rows_h * M;                 // [og][GR][M] the banded products of a group of operators
+  T* Bs = Ys + og * GR * M;                   // [nops][GR][nb] the chunk's band rows
   T* Qs = Bs + nops * GR * nb;             // [Rf][GR] the chunk's source rows
   const int r0 = chunk * GR;
   const int m0 = tile * gmt;
@@ -170,25 +174,27 @@ __device__ __forceinline__ void gram_partial_body(int chunk, int tile, int nchun
   }
   __syncthreads();
   double* out = partial + ((size_t)chunk) * stride;
-  for (int o = 0; o < nops; ++o) {
-    for (int idx = threadIdx.x; idx < GR * M; idx += blockDim.x) {
-      int i = idx / M, n = idx % M;
+  for (int o0 = 0; o0 < nops; o0 += og) {
+    const int go = min(og, nops - o0);
+    if (o0 > 0) __syncthreads();
+    for (int idx = threadIdx.x; idx < go * GR * M; idx += blockDim.x) {
+      const int i = (idx / M) % GR, n = idx % M, o = o0 + idx / (GR * M);
       int gi = r0 + i;
       T acc = 0;
       if (gi < nf) {
         const T* brow = Bs + (o * GR + i) * nb;
         for (int k = 0; k < nb; ++k) acc += brow[k] * Us[(i + k) * M + n];
       }
-      Ys[i * M + n] = acc;
+      Ys[idx] = acc;
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < mt * M; idx += blockDim.x) {
-      int m = m0 + idx / M, n = idx % M;
+    for (int idx = threadIdx.x; idx < go * mt * M; idx += blockDim.x) {
+      const int og_i = idx / (mt * M), m = m0 + (idx / M) % mt, n = idx % M;
+      const T* y = Ys + og_i * GR * M + n;
       T acc = 0;
-      for (int i = 0; i < GR; ++i) acc += Us[(i + hb) * M + m] * Ys[i * M + n];
-      out[((size_t)o * M + m) * M + n] = (double)acc;
+      for (int i = 0; i < GR; ++i) acc += Us[(i + hb) * M + m] * y[i * M];
+      out[((size_t)(o0 + og_i) * M + m) * M + n] = (double)acc;
     }
-    __syncthreads();
   }
   for (int idx = threadIdx.x; idx < Rf * mt; idx += blockDim.x) {
     int r = idx / mt, m = m0 + idx % mt;
@@ -252,9 +258,9 @@ __global__ void gram_partial_kernel(const double* __restrict__ U, int nf, int M,
                                     const double* __restrict__ q, int Rf,
                                     double* __restrict__ partial, int stride, unsigned* ticket,
                                     double* gram, double* h, TermTable tt, GramPtrs gp, int cd,
-                                    double* C, double* c, int gmt, int tail) {
+                                    double* C, double* c, int gmt, int tail, int og) {
   gram_partial_body<T, BF16IN>(blockIdx.x, blockIdx.y, gridDim.x, U, nf, M, hb, opband, nops, q, Rf, partial,
-                               stride, ticket, gram, h, tt, gp, cd, C, c, gmt, tail);
+                               stride, ticket, gram, h, tt, gp, cd, C, c, gmt, tail, og);
 }
 
 // The chunk partials of a dim's Grams added in chunk order and the next dim's
@@ -313,7 +319,7 @@ struct GramAll {
   double* h[TAPS_MAX_DIMS];
   int nf[TAPS_MAX_DIMS], hb[TAPS_MAX_DIMS], nops[TAPS_MAX_DIMS], nchunk[TAPS_MAX_DIMS];
   int cta0[TAPS_MAX_DIMS + 1];
-  int D;
+  int D, og;
 };
 
 __global__ void gram_partial_all_kernel(GramAll ga, int M, int Rf, TermTable tt, GramPtrs gp, int gmt) {
@@ -324,7 +330,7 @@ __global__ void gram_partial_all_kernel(GramAll ga, int M, int Rf, TermTable tt,
   const int nops = ga.nops[d];
   gram_partial_body<double, false>(loc % nchunk, loc / nchunk, nchunk, ga.U[d], ga.nf[d], M, ga.hb[d], ga.band[d],
                                    nops, ga.q[d], Rf, ga.partial[d], nops * M * M + Rf * M, ga.ticket[d],
-                                   ga.gram[d], ga.h[d], tt, gp, -1, nullptr, nullptr, gmt, 1);
+                                   ga.gram[d], ga.h[d], tt, gp, -1, nullptr, nullptr, gmt, 1, ga.og);
 }
 
 // Mode tiles of gmt rows: each tile's last CTA adds its rows' chunk partials, so smaller
@@ -332,6 +338,19 @@ __global__ void gram_partial_all_kernel(GramAll ga, int M, int Rf, TermTable tt,
 // product of its chunk; 4 rows measured fastest up to 32 modes (8 beyond).  The tile
 // height changes no sum's order.  At most 32 tiles (M <= 128).
 static int gram_tile_rows(int M) { return M <= 32 ? 4 : 8; }
+
+// Shared-memory elements of a chunk with the operators in groups of og, and the group: as many
+// operators as 2048 products hold (more only add passes over the same threads), one where the
+// rest already takes most of the 227 KB.  The products of a group are formed between two
+// barriers instead of two barriers per operator: 13 operators of 6 modes, 64 nodes,
+// 22 us one by one and 11 us together.
+static size_t gram_elems(int M, int hb, int nops, int Rf, int og) {
+  return (size_t)(GR + 2 * hb) * M + (size_t)og * GR * M + (size_t)nops * GR * (2 * hb + 1) + (size_t)Rf * GR;
+}
+static int gram_group(int M, int hb, int nops, int Rf) {
+  const int og = std::max(1, std::min(nops, 2048 / (GR * M)));
+  return gram_elems(M, hb, nops, Rf, og) <= 12288 ? og : 1;
+}
 
 static GramPtrs gram_ptrs(const taps_problem* P) {
   GramPtrs gp;
@@ -439,7 +458,7 @@ int taps_refresh_gram_dim(taps_problem* P, const taps_factors* U, int d, int pre
     TAPS_TRY(taps_refresh_gram_dim(P, U, d, precision, -1));
     const int M = U->M;
     int tk = prof_begin(P, TAPS_PROF_COEFF);
-    TAPS_CUDA(taps_launch_pdl(coeff_slots_kernel, dim3((std::max(M * M, P->Rf * M) + 127) / 128), dim3(128), 0, P->stream, P->tt,
+    TAPS_CUDA(taps_launch_pdl(coeff_slots_kernel, dim3(coeff_slots_blocks(P, P->tt.nops[coeff_dim], M)), dim3(128), 0, P->stream, P->tt,
                               gram_ptrs(P), coeff_dim, M, P->d_C, P->d_c));
     prof_end(P, TAPS_PROF_COEFF, tk, (double)P->R * M * M * P->D, 8.0 * ((double)P->R * M * M * P->D));
     P->c0_valid = (coeff_dim == 0);
@@ -453,7 +472,8 @@ int taps_refresh_gram_dim(taps_problem* P, const taps_factors* U, int d, int pre
   int stride = nops * M * M + Rf * M;
   const int gmt = gram_tile_rows(M);
   dim3 grid(nchunk, (M + gmt - 1) / gmt);
-  size_t elems = (size_t)(GR + 2 * hb) * M + (size_t)GR * M + (size_t)nops * GR * (2 * hb + 1) + (size_t)Rf * GR;
+  const int og = gram_group(M, hb, nops, Rf);
+  const size_t elems = gram_elems(M, hb, nops, Rf, og);
   const int nb = 2 * hb + 1;
   double gflops = nops * (2.0 * nb * nf * M + 2.0 * nf * (double)M * M) + 2.0 * Rf * nf * M;
   double gbytes = 8.0 * ((double)nf * M + (double)nops * nf * nb + (double)Rf * nf +
@@ -502,12 +522,12 @@ int taps_refresh_gram_dim(taps_problem* P, const taps_factors* U, int d, int pre
     TAPS_CUDA(taps_launch_pdl(gram_partial_kernel<float, false>, grid, dim3(256), elems * sizeof(float),
                               P->stream, (const double*)U->d_U[d], nf, M, hb, (const double*)P->d_opband[d], nops,
                               (const double*)P->d_q[d], Rf, P->d_partial, stride, P->d_ticket, P->d_gram[d],
-                              P->d_h[d], P->tt, gp, coeff_dim, P->d_C, P->d_c, gmt, 1));
+                              P->d_h[d], P->tt, gp, coeff_dim, P->d_C, P->d_c, gmt, 1, og));
   } else if (precision == TAPS_BF16) {
     TAPS_CUDA(taps_launch_pdl(gram_partial_kernel<float, true>, grid, dim3(256), elems * sizeof(float),
                               P->stream, (const double*)U->d_U[d], nf, M, hb, (const double*)P->d_opband[d], nops,
                               (const double*)P->d_q[d], Rf, P->d_partial, stride, P->d_ticket, P->d_gram[d],
-                              P->d_h[d], P->tt, gp, coeff_dim, P->d_C, P->d_c, gmt, 1));
+                              P->d_h[d], P->tt, gp, coeff_dim, P->d_C, P->d_c, gmt, 1, og));
   } else {
     // FP64: the chunk partials (8-mode tiles: without the tail, fewer tiles recompute
     // the banded products fewer times), then the chunk sums and coefficients spread over
@@ -516,7 +536,8 @@ int taps_refresh_gram_dim(taps_problem* P, const taps_factors* U, int d, int pre
     TAPS_CUDA(taps_launch_pdl(gram_partial_kernel<double, false>, dim3(nchunk, (M + gmt8 - 1) / gmt8), dim3(256),
                               elems * sizeof(double), P->stream, (const double*)U->d_U[d], nf, M, hb,
                               (const double*)P->d_opband[d], nops, (const double*)P->d_q[d], Rf, P->d_partial, stride,
-                              P->d_ticket, P->d_gram[d], P->d_h[d], P->tt, gp, coeff_dim, P->d_C, P->d_c, gmt8, 0));
+                              P->d_ticket, P->d_gram[d], P->d_h[d], P->tt, gp, coeff_dim, P->d_C, P->d_c, gmt8, 0,
+                              og));
     const int nCg = (M * M + 31) / 32, nCh = (Rf * M + 31) / 32;
     TAPS_CUDA(taps_launch_pdl(gram_reduce_coeff_kernel, dim3(nCg + nCh), dim3(32 * std::min(nops, 8)), 0, P->stream,
                               (const double*)P->d_partial, stride, nchunk, M, nops, Rf, P->d_gram[d], P->d_h[d],
@@ -566,11 +587,18 @@ int taps_refresh_grams(taps_problem* P, const taps_factors* U, int precision) {
     ga.nchunk[d] = (nf + GR - 1) / GR;
     ga.cta0[d + 1] = ga.cta0[d] + ga.nchunk[d] * ntile;
     off += (size_t)ga.nchunk[d] * (nops * M * M + Rf * M);
-    elems = std::max(elems, (size_t)(GR + 2 * hb) * M + (size_t)GR * M + (size_t)nops * GR * nb + (size_t)Rf * GR);
     gflops += nops * (2.0 * nb * nf * M + 2.0 * nf * (double)M * M) + 2.0 * Rf * nf * M;
     gbytes += 8.0 * ((double)nf * M + (double)nops * nf * nb + (double)Rf * nf + (double)nops * M * M +
                      (double)Rf * M);
   }
+  int most_ops = 1, most_hb = 0;   // one group size for the launch
+  for (int d = 0; d < P->D; ++d) {
+    most_ops = std::max(most_ops, (int)P->tt.nops[d]);
+    most_hb = std::max(most_hb, P->dims[d]->hb);
+  }
+  ga.og = gram_group(M, most_hb, most_ops, Rf);
+  for (int d = 0; d < P->D; ++d)
+    elems = std::max(elems, gram_elems(M, P->dims[d]->hb, P->tt.nops[d], Rf, ga.og));
   int tk = prof_begin(P, TAPS_PROF_GRAM);
   TAPS_CUDA(taps_launch_pdl(gram_partial_all_kernel, dim3(ga.cta0[P->D]), dim3(256), elems * sizeof(double),
                             P->stream, ga, M, Rf, P->tt, gram_ptrs(P), gmt));
@@ -1176,7 +1204,7 @@ int taps_sweep_setup(int dev, int num_sms, int* coop_blocks, int* ts_most, size_
 static int coefficients(taps_problem* P, int d, int M) {
   int tk = prof_begin(P, TAPS_PROF_COEFF);
   if (P->tt.cs > TAPS_NUM_OPS)
-    TAPS_CUDA(taps_launch_pdl(coeff_slots_kernel, dim3((std::max(M * M, P->Rf * M) + 127) / 128), dim3(128), 0, P->stream, P->tt,
+    TAPS_CUDA(taps_launch_pdl(coeff_slots_kernel, dim3(coeff_slots_blocks(P, P->tt.nops[d], M)), dim3(128), 0, P->stream, P->tt,
                               gram_ptrs(P), d, M, P->d_C, P->d_c));
   else
     TAPS_CUDA(taps_launch_pdl(coeff_kernel, dim3((std::max(M * M, P->Rf * M) + 127) / 128), dim3(128), 0, P->stream, P->tt,
@@ -1551,8 +1579,9 @@ int taps_residual_enqueue(taps_problem* P, const taps_factors* U, int kind, int 
     // then every dim's residual in one launch.
     if (!grams_current) TAPS_TRY(taps_refresh_grams(P, U, TAPS_FP64));
     int tk = prof_begin(P, TAPS_PROF_COEFF);
+    const int most_ops = *std::max_element(P->tt.nops, P->tt.nops + P->D);
     if (P->tt.cs > TAPS_NUM_OPS)
-      TAPS_CUDA(taps_launch_pdl(coeff_all_slots_kernel, dim3((std::max(M * M, P->Rf * M) + 127) / 128, P->D), dim3(128), 0, s,
+      TAPS_CUDA(taps_launch_pdl(coeff_all_slots_kernel, dim3(coeff_slots_blocks(P, most_ops, M), P->D), dim3(128), 0, s,
                                 P->tt, gram_ptrs(P), M, P->d_Call, P->d_call));
     else
       TAPS_CUDA(taps_launch_pdl(coeff_all_kernel, dim3((std::max(M * M, P->Rf * M) + 127) / 128, P->D), dim3(128), 0, s, P->tt,
