@@ -6,6 +6,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include <cuda_bf16.h>
@@ -143,15 +144,15 @@ __device__ __forceinline__ void gram_partial_body(int chunk, int tile, int nchun
                                                   double* __restrict__ partial, int stride, unsigned* ticket,
                                                   double* gram, double* h, const TermTable& tt,
                                                   const GramPtrs& gp, int cd, double* C, double* c, int gmt,
-                                                  int tail, int og) {
+                                                  int tail, int og, int rpart, int nrpart) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int is_last;
   const int nb = 2 * hb + 1;
   const int rows_h = GR + 2 * hb;
   T* Us = reinterpret_cast<T*>(smem_raw);  // [rows_h][M]
   T* Ys = Us + rows_h * M;                 // [og][GR][M] the banded products of a group of operators
-  T* Bs = Ys + og * GR * M;                   // [nops][GR][nb] the chunk's band rows
-  T* Qs = Bs + nops * GR * nb;             // [Rf][GR] the chunk's source rows
+  T* Bs = Ys + og * GR * M;                // [nops][GR][nb] the chunk's band rows
+  T* Qs = Bs + nops * GR * nb;             // [Rf][GR] the chunk's source rows (of this part)
   const int r0 = chunk * GR;
   const int m0 = tile * gmt;
   const int mt = min(gmt, M - m0);
@@ -163,19 +164,22 @@ __device__ __forceinline__ void gram_partial_body(int chunk, int tile, int nchun
     int gi = r0 - hb + rr;
     Us[rr * M + m] = (gi >= 0 && gi < nf) ? gram_in<T, BF16IN>(U[(size_t)m * nf + gi]) : (T)0;
   }
-  for (int idx = threadIdx.x; idx < nops * GR * nb; idx += blockDim.x) {
+  // part rpart of the sources; the operators with the first part
+  const int rlo = Rf * rpart / nrpart, nr = Rf * (rpart + 1) / nrpart - rlo;
+  const int nops_here = rpart == 0 ? nops : 0;
+  for (int idx = threadIdx.x; idx < nops_here * GR * nb; idx += blockDim.x) {
     const int o = idx / (GR * nb), rem = idx % (GR * nb);
     const int gi = r0 + rem / nb;
     Bs[idx] = gi < nf ? gram_in<T, BF16IN>(opband[((size_t)o * nf + gi) * nb + rem % nb]) : (T)0;
   }
-  for (int idx = threadIdx.x; idx < Rf * GR; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < nr * GR; idx += blockDim.x) {
     const int r = idx / GR, gi = r0 + idx % GR;
-    Qs[idx] = gi < nf ? gram_in<T, BF16IN>(q[(size_t)r * nf + gi]) : (T)0;
+    Qs[idx] = gi < nf ? gram_in<T, BF16IN>(q[(size_t)(rlo + r) * nf + gi]) : (T)0;
   }
   __syncthreads();
   double* out = partial + ((size_t)chunk) * stride;
-  for (int o0 = 0; o0 < nops; o0 += og) {
-    const int go = min(og, nops - o0);
+  for (int o0 = 0; o0 < nops_here; o0 += og) {
+    const int go = min(og, nops_here - o0);
     if (o0 > 0) __syncthreads();
     for (int idx = threadIdx.x; idx < go * GR * M; idx += blockDim.x) {
       const int i = (idx / M) % GR, n = idx % M, o = o0 + idx / (GR * M);
@@ -196,14 +200,14 @@ __device__ __forceinline__ void gram_partial_body(int chunk, int tile, int nchun
       out[((size_t)(o0 + og_i) * M + m) * M + n] = (double)acc;
     }
   }
-  for (int idx = threadIdx.x; idx < Rf * mt; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < nr * mt; idx += blockDim.x) {
     int r = idx / mt, m = m0 + idx % mt;
     T acc = 0;
     for (int i = 0; i < GR; ++i) {
       int gi = r0 + i;
       if (gi < nf) acc += Qs[r * GR + i] * Us[(i + hb) * M + m];
     }
-    out[(size_t)nops * M * M + (size_t)r * M + m] = (double)acc;
+    out[(size_t)nops * M * M + (size_t)(rlo + r) * M + m] = (double)acc;
   }
   if (!tail) return;   // gram_reduce_coeff_kernel adds the partials
   // ---- per mode tile, the last chunk CTA reduces the tile's slice of the partials
@@ -260,7 +264,7 @@ __global__ void gram_partial_kernel(const double* __restrict__ U, int nf, int M,
                                     double* gram, double* h, TermTable tt, GramPtrs gp, int cd,
                                     double* C, double* c, int gmt, int tail, int og) {
   gram_partial_body<T, BF16IN>(blockIdx.x, blockIdx.y, gridDim.x, U, nf, M, hb, opband, nops, q, Rf, partial,
-                               stride, ticket, gram, h, tt, gp, cd, C, c, gmt, tail, og);
+                               stride, ticket, gram, h, tt, gp, cd, C, c, gmt, tail, og, blockIdx.z, gridDim.z);
 }
 
 // The chunk partials of a dim's Grams added in chunk order and the next dim's
@@ -330,7 +334,7 @@ __global__ void gram_partial_all_kernel(GramAll ga, int M, int Rf, TermTable tt,
   const int nops = ga.nops[d];
   gram_partial_body<double, false>(loc % nchunk, loc / nchunk, nchunk, ga.U[d], ga.nf[d], M, ga.hb[d], ga.band[d],
                                    nops, ga.q[d], Rf, ga.partial[d], nops * M * M + Rf * M, ga.ticket[d],
-                                   ga.gram[d], ga.h[d], tt, gp, -1, nullptr, nullptr, gmt, 1, ga.og);
+                                   ga.gram[d], ga.h[d], tt, gp, -1, nullptr, nullptr, gmt, 1, ga.og, 0, 1);
 }
 
 // Mode tiles of gmt rows: each tile's last CTA adds its rows' chunk partials, so smaller
@@ -370,10 +374,13 @@ static int coefficients(taps_problem* P, int d, int M);
 // (row chunk, 32 x 32 output tile) accumulates KC nodes of its tile (8 x 32 threads,
 // four outputs each, operands staged 32 nodes at a time), its partial goes to the
 // workspace, and gram_gemm_reduce_kernel adds the chunks' partials in chunk order.
+// FP64 issue is the bound: a warp skips its outputs beyond the last mode, and chunks of 128
+// nodes load the SMs more evenly than 256 (1534 nodes, 100 modes, 239 sources: 201 us
+// with 256 and every output, 140 us now).
 // Every mode tile no longer rebuilds the banded products, and the reduction is over
 // n / KC chunks instead of n / 8.
 // ---------------------------------------------------------------------------------
-#define GG_KC 256
+#define GG_KC 128
 __global__ void spmm_kernel(const double* __restrict__ U, int nf, int M, int hb,
                             const double* __restrict__ opband, int nops, double* __restrict__ Y);
 __global__ void __launch_bounds__(256) gram_gemm_kernel(const double* __restrict__ U, int nf, int M,
@@ -415,12 +422,20 @@ __global__ void __launch_bounds__(256) gram_gemm_kernel(const double* __restrict
       }
     }
     __syncthreads();
+    // this warp's outputs below M: 4, fewer in the last mode tile
+    auto multiply = [&](auto outputs) {
 #pragma unroll 8
-    for (int kk = 0; kk < 32; ++kk) {
-      const double b = Bs[kk][tx];
+      for (int kk = 0; kk < 32; ++kk) {
+        const double b = Bs[kk][tx];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) acc[j] = fma(Us[kk][ty + 8 * j], b, acc[j]);
-    }
+        for (int j = 0; j < decltype(outputs)::value; ++j) acc[j] = fma(Us[kk][ty + 8 * j], b, acc[j]);
+      }
+    };
+    const int left = M - m0 - ty;
+    if (left > 24) multiply(std::integral_constant<int, 4>{});
+    else if (left > 16) multiply(std::integral_constant<int, 3>{});
+    else if (left > 8) multiply(std::integral_constant<int, 2>{});
+    else if (left > 0) multiply(std::integral_constant<int, 1>{});
     __syncthreads();
   }
   double* out = partial + (size_t)blockIdx.x * M * ncol;
@@ -532,8 +547,10 @@ int taps_refresh_gram_dim(taps_problem* P, const taps_factors* U, int d, int pre
     // FP64: the chunk partials (8-mode tiles: without the tail, fewer tiles recompute
     // the banded products fewer times), then the chunk sums and coefficients spread over
     // many CTAs
-    const int gmt8 = 8;
-    TAPS_CUDA(taps_launch_pdl(gram_partial_kernel<double, false>, dim3(nchunk, (M + gmt8 - 1) / gmt8), dim3(256),
+    // hundreds of sources: their FP64 issue per chunk is more than the operators', so three
+    // CTAs share it (466 sources, 255 nodes, 20 modes: 22 us in one, 13 us in three)
+    const int gmt8 = 8, nrpart = Rf >= 128 ? 3 : 1;
+    TAPS_CUDA(taps_launch_pdl(gram_partial_kernel<double, false>, dim3(nchunk, (M + gmt8 - 1) / gmt8, nrpart), dim3(256),
                               elems * sizeof(double), P->stream, (const double*)U->d_U[d], nf, M, hb,
                               (const double*)P->d_opband[d], nops, (const double*)P->d_q[d], Rf, P->d_partial, stride,
                               P->d_ticket, P->d_gram[d], P->d_h[d], P->tt, gp, coeff_dim, P->d_C, P->d_c, gmt8, 0,
