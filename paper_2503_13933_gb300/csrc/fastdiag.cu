@@ -836,8 +836,32 @@ __global__ void __launch_bounds__(128) fd_rhs_kernel(const double* __restrict__ 
       Rf, [&](int r) { return q[(size_t)r * nf + i]; }, [&](int r) { return c[(size_t)r * M + m]; });
 }
 
-int taps_rhs(const double* q, const double* c, int Rf, int n, int M, double* F, cudaStream_t s) {
-  fd_rhs_kernel<<<(unsigned)(((long long)n * M + 127) / 128), 128, 0, s>>>(q, c, Rf, n, M, F);
+// The same with the sum over r in four parts, one per warp of a CTA of 32 entries.
+__global__ void __launch_bounds__(128) fd_rhs_split_kernel(const double* __restrict__ q, const double* __restrict__ c,
+                                                           int Rf, int nf, int M, double* __restrict__ F) {
+  __shared__ double part[4][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const long long idx = (long long)blockIdx.x * 32 + lane;
+  const bool in = idx < (long long)nf * M;
+  const int i = in ? (int)(idx / M) : 0, m = in ? (int)(idx % M) : 0;
+  const int r0 = Rf * w / 4, r1 = Rf * (w + 1) / 4;
+  const double *qi = q + (size_t)r0 * nf + i, *cm = c + (size_t)r0 * M + m;
+  part[w][lane] = taps_fma_chain<16>(
+      r1 - r0, [&](int r) { return qi[(size_t)r * nf]; }, [&](int r) { return cm[(size_t)r * M]; });
+  __syncthreads();
+  if (w == 0 && in) F[idx] = (part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane]);
+}
+
+// The chain of R_f dependent FMAs bounds a moving source's hundreds of terms while the entries
+// leave most sub-partitions idle; beyond a warp per sub-partition the FP64 issue does, and
+// splitting the chain gives nothing.  466 terms, 255 nodes of 20 modes: 47 us as one
+// chain, 16 us in four; 239 terms, 1534 nodes of 100 modes: 95 us as one chain.
+int taps_rhs(const double* q, const double* c, int Rf, int n, int M, double* F, int num_sms, cudaStream_t s) {
+  const long long nM = (long long)n * M;
+  if (Rf >= 128 && nM <= 128ll * num_sms)
+    fd_rhs_split_kernel<<<(unsigned)((nM + 31) / 32), 128, 0, s>>>(q, c, Rf, n, M, F);
+  else
+    fd_rhs_kernel<<<(unsigned)((nM + 127) / 128), 128, 0, s>>>(q, c, Rf, n, M, F);
   TAPS_CUDA(cudaGetLastError());
   return TAPS_OK;
 }
@@ -912,6 +936,98 @@ __global__ void __launch_bounds__(RG_WARPS * 32) fd_rowgemm_kernel(const double*
     }
     __syncthreads();
   }
+}
+
+// The same product as a tiled contraction for many rows and modes: a CTA takes 32 rows (lane =
+// row) of four modes (warp = mode, so that a mode count that is no multiple of the tile wastes
+// no FP64 issue), 32 columns of Mat at a time through two shared buffers, the next ones loaded
+// while these are multiplied.  Each tile is four chains of 8, and the tiles are added in pairs up
+// to eight, so that an entry's rounding stays that of the row kernel's short sums (6.9e-15 against
+// 6.8e-15 rms over 1534 normal products).  The row kernel pays a butterfly
+// per row and 32 modes and an L1 line per lane and operand; FP64 issue is the bound of this one.
+// 1534 rows of 100 modes: 621 us with a CTA per row, 461 us.
+#define FM_TILE 32
+#define FM_WARPS 4
+__global__ void __launch_bounds__(FM_WARPS * 32) fd_matmul_kernel(const double* __restrict__ Mat,
+                                                                  const double* __restrict__ In, int n, int M,
+                                                                  double* __restrict__ Out, int colmajor,
+                                                                  double* __restrict__ Save) {
+  __shared__ double As[2][FM_TILE][FM_TILE + 1];   // [column of Mat][row]
+  __shared__ double Bs[2][FM_TILE][FM_WARPS];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int i0 = blockIdx.x * FM_TILE, m0 = blockIdx.y * FM_WARPS;
+  const int i = i0 + lane, m = m0 + warp;
+  double ra[FM_TILE / FM_WARPS], rb;
+  auto load = [&](int k0) {
+    const int k = k0 + lane;
+#pragma unroll
+    for (int e = 0; e < FM_TILE / FM_WARPS; ++e) {
+      const int r = i0 + warp + FM_WARPS * e;
+      ra[e] = (r < n && k < n) ? Mat[(size_t)r * n + k] : 0.0;
+    }
+    const int kb = k0 + tid / FM_WARPS, mb = m0 + tid % FM_WARPS;
+    rb = (kb < n && mb < M) ? In[(size_t)kb * M + mb] : 0.0;
+  };
+  taps_pdl_wait();
+  load(0);
+  double sum = 0.0, one = 0.0, two = 0.0, four = 0.0;
+  int t = 0;
+  for (int k0 = 0; k0 < n; k0 += FM_TILE, ++t) {
+    const int cur = t & 1;
+#pragma unroll
+    for (int e = 0; e < FM_TILE / FM_WARPS; ++e) As[cur][lane][warp + FM_WARPS * e] = ra[e];
+    Bs[cur][tid / FM_WARPS][tid % FM_WARPS] = rb;
+    __syncthreads();   // the other buffer's readers are past it as well
+    if (k0 + FM_TILE < n) load(k0 + FM_TILE);
+    if (m < M) {
+      double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+      for (int k = 0; k < FM_TILE / 4; ++k)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int kc = k + c * (FM_TILE / 4);
+          a[c] = fma(As[cur][kc][lane], Bs[cur][kc][warp], a[c]);
+        }
+      double x = (a[0] + a[1]) + (a[2] + a[3]);
+      // pairwise up to eight tiles
+      if (!(t & 1)) one = x;
+      else {
+        x += one;
+        if (!(t & 2)) two = x;
+        else {
+          x += two;
+          if (!(t & 4)) four = x;
+          else sum += x + four;
+        }
+      }
+    }
+  }
+  if (m >= M || i >= n) return;
+  if (t & 4) sum += four;
+  if (t & 2) sum += two;
+  if (t & 1) sum += one;
+  if (!colmajor) {
+    Out[(size_t)i * M + m] = sum;
+    return;
+  }
+  double* o = Out + (size_t)m * n + i;
+  if (Save) Save[(size_t)m * n + i] = *o;
+  *o = sum;
+}
+
+// The tiled product beyond 32 modes, where the row kernel takes more than one pass over Mat and
+// its lanes' operands lie further apart (64 modes: 9.6 and 5.0 us for 12 rows, 25 and 17 for 254,
+// 46 and 34 for 382, 87 and 51 for 606; 40 modes: 191 and 140 us for 1214 rows).  Up to 32 modes
+// its tiles are too few and their chains the longer ones (254 rows of 30 modes: 10.6 and 16.8 us).
+static int fd_transform(const double* Mat, const double* In, int n, int M, double* Out, int colmajor, double* Save,
+                        cudaStream_t s) {
+  if (M > 32)
+    TAPS_CUDA(taps_launch_pdl(fd_matmul_kernel, dim3((n + FM_TILE - 1) / FM_TILE, (M + FM_WARPS - 1) / FM_WARPS),
+                              dim3(FM_WARPS * 32), 0, s, Mat, In, n, M, Out, colmajor, Save));
+  else
+    TAPS_CUDA(taps_launch_pdl(fd_rowgemm_kernel, dim3(n), dim3(RG_WARPS * 32), 0, s, Mat, In, n, M, Out, colmajor,
+                              Save));
+  return TAPS_OK;
 }
 
 // One warp per node i, M <= 32: lane r holds row r of (mu_i C_A + C_B | g_i) in
@@ -1501,7 +1617,7 @@ int taps_fd_solve(taps_problem* P, taps_factors* U, int d, int precision) {
                               slotA >= 0 ? (const double*)E->mu : nullptr, (const double*)P->d_pq[d],
                               (const double*)P->d_c, P->Rf, n, M, Y, P->d_status));
   } else {
-    TAPS_TRY(taps_rhs(P->d_pq[d], P->d_c, P->Rf, n, M, G, s));
+    TAPS_TRY(taps_rhs(P->d_pq[d], P->d_c, P->Rf, n, M, G, P->num_sms, s));
     if (M <= 32)
       fd_small_solve_warp_kernel<<<n, 32, 0, s>>>(CA, CB, slotA >= 0 ? E->mu : nullptr, G, n, M, Y,
                                                   P->d_status, 1);
@@ -1525,8 +1641,7 @@ int taps_fd_solve(taps_problem* P, taps_factors* U, int d, int precision) {
            8.0 * ((double)P->Rf * n + 2.0 * MM + (double)nM));
   // back to the nodal basis; the previous factor goes to d_Uold for the change norm
   tk = prof_begin(P, TAPS_PROF_FD_TRANSFORM);
-  TAPS_CUDA(taps_launch_pdl(fd_rowgemm_kernel, dim3(n), dim3(RG_WARPS * 32), 0, s, (const double*)E->Phi,
-                            (const double*)Y, n, M, U->d_U[d], 1, P->d_Uold));
+  TAPS_TRY(fd_transform(E->Phi, Y, n, M, U->d_U[d], 1, P->d_Uold, s));
   prof_end(P, TAPS_PROF_FD_TRANSFORM, tk, 2.0 * (double)n * n * M, 8.0 * ((double)n * n + 3.0 * nM));
   TAPS_CUDA(cudaGetLastError());
   return TAPS_OK;
@@ -1543,8 +1658,7 @@ int taps_fd_lookup(taps_problem* P, int d, int opA, int opB, const FdEntry** out
 // Out = Phi Y in the factor layout (Y n x M row-major), the previous factor into Save.
 int taps_fd_to_nodal(taps_problem* P, const FdEntry* E, const double* Y, int n, int M, double* Out, double* Save) {
   int tk = prof_begin(P, TAPS_PROF_FD_TRANSFORM);
-  TAPS_CUDA(taps_launch_pdl(fd_rowgemm_kernel, dim3(n), dim3(RG_WARPS * 32), 0, P->stream, (const double*)E->Phi,
-                            Y, n, M, Out, 1, Save));
+  TAPS_TRY(fd_transform(E->Phi, Y, n, M, Out, 1, Save, P->stream));
   prof_end(P, TAPS_PROF_FD_TRANSFORM, tk, 2.0 * (double)n * n * M, 8.0 * ((double)n * n + 3.0 * (double)n * M));
   TAPS_CUDA(cudaGetLastError());
   return TAPS_OK;

@@ -345,7 +345,7 @@ int taps_fdw_solve(taps_problem* P, taps_factors* U, int d) {
   int tk = prof_begin(P, TAPS_PROF_FASTDIAG);
   // g_i for every node first: inside the node's one warp, hundreds of source terms' loads were
   // most of its time
-  TAPS_TRY(taps_rhs(P->d_pq[d], P->d_c, P->Rf, n, M, P->d_Y, s));
+  TAPS_TRY(taps_rhs(P->d_pq[d], P->d_c, P->Rf, n, M, P->d_Y, P->num_sms, s));
   fdw_node_kernel<<<n, 128, 0, s>>>(P->d_C + (size_t)sa * MM, P->d_C + (size_t)sb * MM, E->mu, P->d_Y, n, M,
                                     P->num_sms, X, w, P->d_status);
   fdw_reduce_kernel<<<dim3((M * M + 31) / 32, nbnd == 2 ? 5 : 2), 32, 0, s>>>(X, w, E->Phi, corner0, corner1, n, M,

@@ -1657,8 +1657,8 @@ int taps_md_setup(int maxsm) {
 template <int HB>
 static cudaError_t md_band_launch(const double* bx, const double* by, const double* lam, const double* q,
                                   const double* cw, int Rf, int n, int M, double* Fw, double* scratch, double* Z,
-                                  int* status, cudaStream_t s) {
-  if (taps_rhs(q, cw, Rf, n, M, Fw, s) != TAPS_OK) return cudaErrorLaunchFailure;   // (F W)_j
+                                  int* status, int num_sms, cudaStream_t s) {
+  if (taps_rhs(q, cw, Rf, n, M, Fw, num_sms, s) != TAPS_OK) return cudaErrorLaunchFailure;   // (F W)_j
   md_band_kernel<HB><<<M, 32, 0, s>>>(bx, by, lam, Fw, n, M, scratch, Z, status);
   return cudaGetLastError();
 }
@@ -1774,12 +1774,13 @@ int taps_md_solve(taps_problem* P, taps_factors* U, int d) {
     md_cw_kernel<<<(unsigned)((rm + 255) / 256), 256, 0, s>>>(P->d_c, Wm, Rf, M, cw);
   }
   cudaError_t ce = cudaSuccess;
+  const int sms = P->num_sms;
   switch (hb) {
-    case 1: ce = md_band_launch<1>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, s); break;
-    case 2: ce = md_band_launch<2>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, s); break;
-    case 3: ce = md_band_launch<3>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, s); break;
-    case 4: ce = md_band_launch<4>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, s); break;
-    default: ce = md_band_launch<5>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, s); break;
+    case 1: ce = md_band_launch<1>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, sms, s); break;
+    case 2: ce = md_band_launch<2>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, sms, s); break;
+    case 3: ce = md_band_launch<3>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, sms, s); break;
+    case 4: ce = md_band_launch<4>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, sms, s); break;
+    default: ce = md_band_launch<5>(bx, by, lam, P->d_q[d], cw, Rf, n, M, Fw, scratch, Z, P->d_status, sms, s); break;
   }
   TAPS_CUDA(ce);
   const long long nM = (long long)n * M;

@@ -466,6 +466,6 @@ size_t taps_ts_scratch_doubles(int hb, int M);
 int taps_ts_solve(taps_problem* P, taps_factors* U, int d, int nc);
 int taps_fd_eligible(const taps_problem* P, int d, int* slotA, int* slotB);
 // F[i][m] = sum_r q[r][i] c[r][m] (q [Rf][n], c [Rf][M], F [n][M]).
-int taps_rhs(const double* q, const double* c, int Rf, int n, int M, double* F, cudaStream_t s);
+int taps_rhs(const double* q, const double* c, int Rf, int n, int M, double* F, int num_sms, cudaStream_t s);
 int taps_fd_solve(taps_problem* P, taps_factors* U, int d, int precision);
 void taps_fd_release(taps_dim* dm);
