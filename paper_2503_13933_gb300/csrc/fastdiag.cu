@@ -392,6 +392,149 @@ __global__ void __launch_bounds__(TDS_THREADS)
   }
 }
 
+// The same with the rows of S in the shared memory of the whole chip, one cooperative launch: CTA
+// r keeps rows r, r + G, ...  One grid barrier per step: a pass over the own rows applies the last
+// step's update, multiplies by the new reflector and publishes p and row k + 1 (the next column,
+// before this step's update) in global memory; after the barrier every CTA forms w and the
+// updated column from them, and from that the next reflector.  Two copies of the published
+// vectors, so that a CTA ahead never overwrites what another still reads.  The chain of a step
+// (barrier, two block sums, the reflector's scalars) is the bound; the cluster version reads and
+// writes S in L2 twice a step on 16 SMs.  1534 nodes: 128 ms on a cluster, 21.7 ms here.
+#define TDG_THREADS 512
+#define TDG_PER 4   // entries of a column to a thread: n <= TDG_THREADS * TDG_PER
+__global__ void __launch_bounds__(TDG_THREADS)
+    fd_tridiag_grid_kernel(const double* __restrict__ A, double* __restrict__ V, double* __restrict__ beta,
+                           double* __restrict__ d, double* __restrict__ e, int n, double* xch, unsigned* bar,
+                           int* status) {
+  extern __shared__ double tsm[];   // two reflectors [2][n] | w [n] | own rows [nr][n]
+  __shared__ double red[TDG_THREADS / 32], sc[4];
+  const int G = gridDim.x, rank = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = TDG_THREADS / 32;
+  double *v = tsm, *vn = tsm + n, *ws = tsm + 2 * n, *rows = tsm + 3 * n;
+  const int nr = rank < n ? (n - rank + G - 1) / G : 0;   // rows rank + G l, l < nr
+  for (long long idx = tid; idx < (long long)nr * n; idx += TDG_THREADS) {
+    const int l = (int)(idx / n), j = (int)(idx % n);
+    rows[(size_t)l * n + j] = A[(size_t)(rank + G * l) * n + j];
+  }
+  double x[TDG_PER];   // row k from its diagonal on: entries tid + TDG_THREADS j
+#pragma unroll
+  for (int j = 0; j < TDG_PER; ++j) {
+    const int t = tid + TDG_THREADS * j;
+    x[j] = t < n ? A[t] : 0.0;
+  }
+  // sum over the block of one value per thread of the first `count`; warp 0 holds it
+  auto partial_sum = [&](double y, int count) {
+    if (warp * 32 < count) {
+      y = warp_sum(y);
+      if (lane == 0) red[warp] = y;
+    } else if (lane == 0) {
+      red[warp] = 0.0;
+    }
+    __syncthreads();
+    return warp == 0 ? warp_sum(lane < nwarps ? red[lane] : 0.0) : 0.0;
+  };
+  // the reflector of step k from row k in x: vn, sc[1] = alpha, sc[2] = beta; zero for a zero column
+  auto reflect = [&](int k) {
+    const int len = n - k - 1;
+    double s2 = 0.0;
+#pragma unroll
+    for (int j = 0; j < TDG_PER; ++j) {
+      const int t = tid + TDG_THREADS * j;
+      if (t >= 1 && t <= len) {
+        vn[t - 1] = x[j];
+        s2 = fma(x[j], x[j], s2);
+      }
+    }
+    if (tid == 1) sc[3] = x[0];
+    s2 = partial_sum(s2, len + 1);
+    if (tid == 0) {
+      double al = 0.0, v0 = 0.0, bk = 0.0;
+      if (s2 != 0.0) {
+        const double x0 = sc[3];
+        al = -copysign(sqrt(s2), x0);
+        v0 = x0 - al;
+        bk = 2.0 / (s2 - x0 * x0 + v0 * v0);
+      }
+      vn[0] = v0;
+      sc[1] = al;
+      sc[2] = bk;
+      if (rank == 0) {
+        d[k] = x[0];
+        e[k] = al;
+        beta[k] = bk;
+      }
+    }
+    __syncthreads();
+    if (rank == 0)
+      for (int t = tid; t < len; t += TDG_THREADS) V[(size_t)k * n + k + 1 + t] = vn[t];
+  };
+  reflect(0);   // its barriers also order the rows' loads
+  for (int k = 0; k + 2 < n; ++k) {
+    const int len = n - k - 1;
+    const double bk = sc[2];
+    double* pbuf = xch + (size_t)(k & 1) * 2 * n;
+    double* rbuf = pbuf + n;
+    for (int l = (k + 1 - rank + G - 1) / G + warp; l < nr; l += nwarps) {
+      const int i = rank + G * l;
+      double* row = rows + (size_t)l * n + (k + 1);
+      const double vi = k > 0 ? v[i - k] : 0.0, wi = k > 0 ? ws[i - k] : 0.0;
+      double acc = 0.0;
+#pragma unroll 4
+      for (int t = lane; t < len; t += 32) {
+        double y = row[t];
+        if (k > 0) {
+          y = fma(-wi, v[t + 1], fma(-vi, ws[t + 1], y));
+          row[t] = y;
+        }
+        if (i == k + 1) rbuf[t] = y;
+        acc = fma(y, vn[t], acc);
+      }
+      acc = warp_sum(acc);
+      if (lane == 0) pbuf[i - k - 1] = bk * acc;
+    }
+    grid_barrier(bar, status, G);
+    double* sw = v;
+    v = vn;
+    vn = sw;
+    double p[TDG_PER], pv = 0.0;
+    const double p0 = __ldcg(pbuf);
+#pragma unroll
+    for (int j = 0; j < TDG_PER; ++j) {
+      const int t = tid + TDG_THREADS * j;
+      p[j] = t < len ? __ldcg(pbuf + t) : 0.0;
+      x[j] = t < len ? __ldcg(rbuf + t) : 0.0;
+    }
+#pragma unroll
+    for (int j = 0; j < TDG_PER; ++j) {
+      const int t = tid + TDG_THREADS * j;
+      if (t < len) pv = fma(p[j], v[t], pv);
+    }
+    pv = partial_sum(pv, len);
+    if (tid == 0) sc[0] = 0.5 * bk * pv;
+    __syncthreads();
+    const double Kc = sc[0], v0 = v[0], w0 = fma(-Kc, v0, p0);
+#pragma unroll
+    for (int j = 0; j < TDG_PER; ++j) {
+      const int t = tid + TDG_THREADS * j;
+      if (t < len) {
+        const double vt = v[t], wt = fma(-Kc, vt, p[j]);
+        ws[t] = wt;
+        x[j] = fma(-w0, vt, fma(-v0, wt, x[j]));   // the update of row k + 1, as its owner forms it
+      }
+    }
+    if (k + 3 < n) reflect(k + 1);
+  }
+  // the last two rows: row n - 2 in x; the last diagonal entry from its owner
+  __syncthreads();
+  if (rank == 0 && tid < 2) {
+    (tid == 0 ? d : e)[n - 2] = x[0];
+    beta[n - 2 + tid] = 0.0;
+    if (tid == 1) e[n - 1] = 0.0;
+  }
+  if ((n - 1) % G == rank && tid == 0)
+    d[n - 1] = fma(-ws[1], v[1], fma(-v[1], ws[1], rows[(size_t)((n - 1) / G) * n + n - 1]));
+}
+
 // ---------------------------------------------------------------------------------
 // Eigenvalues of the symmetric tridiagonal T (diagonal d, off-diagonal e) by Sturm-count
 // multisection: warp k finds the k-th smallest eigenvalue.  Each lane counts the
@@ -476,11 +619,17 @@ __global__ void fd_bisect_kernel(const double* __restrict__ d, const double* __r
 // Eigenvectors of T by inverse iteration: thread k factors T - lam_k I by Gaussian
 // elimination with partial pivoting (U has two super-diagonals) and solves three times
 // from a fixed start vector, normalising after each solve.  Eigenvalues closer than
-// 1e-5 ||T|| form a cluster, handled in order by the thread of its first member, each
-// iterate orthogonalised against the members already done (modified Gram-Schmidt).
+// FD_CLUSTER ||T|| form a cluster, handled in order by the thread of its first member, each
+// iterate orthogonalised against the members already done (modified Gram-Schmidt).  Vectors
+// iterated independently are orthogonal to a few eps ||T|| / gap (1.8e-11 at a gap of
+// 3e-7 ||T||), which the orthogonalisation step below squares, so the limit lies where that is
+// far under eps; the ends of a stiffness pencil's spectrum have gaps of ~2 / n^2 ||T||, and a
+// limit of 1e-5 ||T|| made serial clusters of them from 500 nodes on (1532 nodes:
+// 95 ms, 11.5 ms now).
 // Z is n x n row-major (column k = eigenvector k); W holds five n x n arrays laid out
 // [array][row][k] so that neighbouring threads touch neighbouring words.
 // ---------------------------------------------------------------------------------
+#define FD_CLUSTER 3e-7
 __global__ void fd_invit_kernel(const double* __restrict__ d, const double* __restrict__ e,
                                 const double* __restrict__ lam, int n, double* __restrict__ Z,
                                 double* __restrict__ W) {
@@ -490,7 +639,7 @@ __global__ void fd_invit_kernel(const double* __restrict__ d, const double* __re
   for (int i = 0; i < n; ++i)
     tnorm = fmax(tnorm, fabs(d[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0) + (i + 1 < n ? fabs(e[i]) : 0.0));
   if (!(tnorm > 0.0)) tnorm = 1.0;
-  const double ctol = 1e-5 * tnorm;
+  const double ctol = FD_CLUSTER * tnorm;
   if (k0 > 0 && lam[k0] - lam[k0 - 1] <= ctol) return;   // not the first member of its cluster
   int k1 = k0;
   while (k1 + 1 < n && lam[k1 + 1] - lam[k1] <= ctol) ++k1;
@@ -571,19 +720,23 @@ __global__ void fd_invit_kernel(const double* __restrict__ d, const double* __re
 }
 
 // The same with T, the factors and the iterate in shared memory: IV_COLS eigenvectors to a CTA
-// of one warp.  The passes are chains over the nodes whose global-memory arrays, written and
-// read back by the same thread, were most of their time (254 nodes: 1055 us).
-#define IV_COLS 8
-static size_t iv_smem(int n) { return sizeof(double) * (2 * (size_t)n + 5 * (size_t)n * IV_COLS) + (size_t)n * IV_COLS; }
+// of one warp, as many of 8, 4, 2, 1 as fit (n <= ~820, 1560, 2820, 4770).  The passes are chains over the nodes whose global-memory arrays, written and
+// read back by the same thread, were most of their time (254 nodes: 1055 us;
+// 1534 nodes, 4 to a CTA: 157 ms on global arrays, 95 ms here, 11.5 ms with
+// the narrower clusters).
+static size_t iv_smem(int n, int cols) {
+  return sizeof(double) * (2 * (size_t)n + 4 * (size_t)n * cols) + (size_t)n * cols;
+}
 
+template <int IV_COLS>
 __global__ void __launch_bounds__(32) fd_invit_smem_kernel(const double* __restrict__ dg, const double* __restrict__ eg,
                                                            const double* __restrict__ lam, int n,
                                                            double* __restrict__ Z) {
   extern __shared__ double ism[];
   double* d = ism;
   double* e = ism + n;
-  double* W = ism + 2 * n;                         // [4][n][IV_COLS]: 1/U0, U1, U2, multiplier
-  double* z = W + 4 * (size_t)n * IV_COLS;         // [n][IV_COLS]
+  double* W = ism + 2 * n;                         // [3][n][IV_COLS]: 1/U0, U1, multiplier
+  double* z = W + 3 * (size_t)n * IV_COLS;         // [n][IV_COLS]
   unsigned char* swap = reinterpret_cast<unsigned char*>(z + (size_t)n * IV_COLS);
   const int l = threadIdx.x;
   for (int i = l; i < n; i += 32) {
@@ -597,7 +750,7 @@ __global__ void __launch_bounds__(32) fd_invit_smem_kernel(const double* __restr
   for (int i = 0; i < n; ++i)
     tnorm = fmax(tnorm, fabs(d[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0) + (i + 1 < n ? fabs(e[i]) : 0.0));
   if (!(tnorm > 0.0)) tnorm = 1.0;
-  const double ctol = 1e-5 * tnorm;
+  const double ctol = FD_CLUSTER * tnorm;
   if (k0 > 0 && lam[k0] - lam[k0 - 1] <= ctol) return;   // not the first member of its cluster
   int k1 = k0;
   while (k1 + 1 < n && lam[k1 + 1] - lam[k1] <= ctol) ++k1;
@@ -618,8 +771,7 @@ __global__ void __launch_bounds__(32) fd_invit_smem_kernel(const double* __restr
       const double m = num / den;
       WA(0, i) = 1.0 / den;
       WA(1, i) = keep ? bi : an;
-      WA(2, i) = keep ? 0.0 : bn;
-      WA(3, i) = m;
+      WA(2, i) = m;
       SW(i) = keep ? 0 : 1;
       const double upper = keep ? bi : an;
       ai = (keep ? an : bi) - m * upper;
@@ -628,7 +780,7 @@ __global__ void __launch_bounds__(32) fd_invit_smem_kernel(const double* __restr
     if (ai == 0.0) ai = tiny;
     WA(0, n - 1) = 1.0 / ai;
     WA(1, n - 1) = 0.0;   // the last row has no super-diagonals
-    WA(2, n - 1) = 0.0;
+    SW(n - 1) = 0;
     for (int i = 0; i < n; ++i) ZC(i) = 1.0 + 0.5 * sin(0.7 * i + 1.3 * k);
     for (int it = 0; it < 3; ++it) {
       double yi = ZC(0);
@@ -641,13 +793,14 @@ __global__ void __launch_bounds__(32) fd_invit_smem_kernel(const double* __restr
           yn = t;
         }
         ZC(i) = yi;
-        yi = yn - WA(3, i) * yi;
+        yi = yn - WA(2, i) * yi;
       }
       ZC(n - 1) = yi;
       double z1 = 0.0, z2 = 0.0;
 #pragma unroll 4
       for (int i = n - 1; i >= 0; --i) {
-        const double zi = (ZC(i) - WA(1, i) * z1 - WA(2, i) * z2) * WA(0, i);
+        const double u2 = SW(i) && i + 2 < n ? e[i + 1] : 0.0;   // filled in by an exchange of rows
+        const double zi = (ZC(i) - WA(1, i) * z1 - u2 * z2) * WA(0, i);
         ZC(i) = zi;
         z2 = z1;
         z1 = zi;
@@ -1380,18 +1533,41 @@ static cudaError_t td_launch(void (*fn)(Args...), int threads, size_t smem, cuda
   return cudaLaunchKernelEx(&cfg, fn, args...);
 }
 
-// The tridiagonalisation of S (n x n in A) on one cluster: S in distributed shared
-// memory when its rows fit, else in global memory.
+// Whether every SM can hold a CTA of the whole-chip tridiagonalisation.
+static bool td_grid_ok(size_t smem, int maxsm) {
+  int per_sm = 0;
+  if (taps_allow_dyn_smem((const void*)fd_tridiag_grid_kernel, maxsm) != TAPS_OK ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fd_tridiag_grid_kernel, TDG_THREADS, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return per_sm > 0;
+}
+
+// The tridiagonalisation of S (n x n in A): S in a cluster's distributed shared memory up to
+// TD_CLUSTER_MOST nodes, where its cheaper barriers win, then in the shared memory of all num_sms
+// SMs while its rows fit (152: n <= ~1820), else in global memory.  Cluster and chip: 1.75 and
+// 2.34 ms for 254 nodes, 3.55 and 3.69 for 382, 6.28 and 5.21 for 510, 10.4 and 6.78 for 638.
+// xch: 4 n doubles and two words of workspace.
+#define TD_CLUSTER_MOST 448
 static int td_run(double* A, double* V, double* tmp, double* bt, double* dd, double* ee, int n, int maxsm,
-                  cudaStream_t s) {
+                  int num_sms, double* xch, int* status, cudaStream_t s) {
   const size_t dsm16 = sizeof(double) * ((size_t)((n + 15) / 16) * n + 3 * (size_t)n);
   const size_t dsm8 = sizeof(double) * ((size_t)((n + 7) / 8) * n + 3 * (size_t)n);
   const size_t gsm = sizeof(double) * 3 * (size_t)n;
+  const size_t grd = sizeof(double) * ((size_t)((n + num_sms - 1) / num_sms) * n + 3 * (size_t)n);
   cudaError_t ce;
-  if (dsm16 + 1024 <= (size_t)maxsm && td_cluster_ok<16>((const void*)fd_tridiag_dsmem_kernel<16>, dsm16, TDS_THREADS)) {
+  const bool small = n <= TD_CLUSTER_MOST || grd + 1024 > (size_t)maxsm || n > TDG_THREADS * TDG_PER;
+  if (small && dsm16 + 1024 <= (size_t)maxsm && td_cluster_ok<16>((const void*)fd_tridiag_dsmem_kernel<16>, dsm16, TDS_THREADS)) {
     ce = td_launch<16>(fd_tridiag_dsmem_kernel<16>, TDS_THREADS, dsm16, s, (const double*)A, V, bt, dd, ee, n);
-  } else if (dsm8 + 1024 <= (size_t)maxsm && td_cluster_ok<8>((const void*)fd_tridiag_dsmem_kernel<8>, dsm8, TDS_THREADS)) {
+  } else if (small && dsm8 + 1024 <= (size_t)maxsm && td_cluster_ok<8>((const void*)fd_tridiag_dsmem_kernel<8>, dsm8, TDS_THREADS)) {
     ce = td_launch<8>(fd_tridiag_dsmem_kernel<8>, TDS_THREADS, dsm8, s, (const double*)A, V, bt, dd, ee, n);
+  } else if (!small && td_grid_ok(grd, maxsm)) {
+    unsigned* bar = reinterpret_cast<unsigned*>(xch + 4 * (size_t)n);
+    TAPS_CUDA(cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), s));
+    const double* Ac = A;
+    void* args[] = {&Ac, &V, &bt, &dd, &ee, &n, &xch, &bar, &status};
+    ce = cudaLaunchCooperativeKernel((const void*)fd_tridiag_grid_kernel, dim3(num_sms), dim3(TDG_THREADS), args, grd, s);
   } else if (td_cluster_ok<16>((const void*)fd_tridiag_kernel<16>, gsm, TD_THREADS)) {
     ce = td_launch<16>(fd_tridiag_kernel<16>, TD_THREADS, gsm, s, A, V, tmp, bt, dd, ee, n);
   } else {
@@ -1451,6 +1627,13 @@ static int fd_cholesky(const double* band, double* B, int n, int hb, double* lin
     fd_cholesky_global_kernel<<<1, FD_THREADS, 0, s>>>(B, n, hb, linv, status);
   }
   TAPS_CUDA(cudaGetLastError());
+  return TAPS_OK;
+}
+
+template <int C>
+static int iv_launch(const double* dd, const double* ee, const double* lam, int n, double* Z, int maxsm, cudaStream_t s) {
+  TAPS_TRY(taps_allow_dyn_smem((const void*)fd_invit_smem_kernel<C>, maxsm));
+  fd_invit_smem_kernel<C><<<(n + C - 1) / C, 32, iv_smem(n, C), s>>>(dd, ee, lam, n, Z);
   return TAPS_OK;
 }
 
@@ -1518,18 +1701,22 @@ static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, FdEntry**
       if ((st = fd_lsolve(B, linv, V, n, dm->hb, 1, W, s)) != TAPS_OK) break;
       fd_symmetrize_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(W, n, A);
       if (cudaMemsetAsync(V, 0, sizeof(double) * nn, s) != cudaSuccess) { st = TAPS_ERR_CUDA; break; }
-      if ((st = td_run(A, V, T->tmp, T->bt, T->dd, T->ee, n, maxsm_optin, s)) != TAPS_OK) break;
+      if ((st = td_run(A, V, T->tmp, T->bt, T->dd, T->ee, n, maxsm_optin, P->num_sms, W, P->d_status, s)) != TAPS_OK) break;
       // eigenvalues (warp each), eigenvectors (thread each), back-transform (warp each),
       // all into A, which the tridiagonalisation no longer needs
       // two warps per CTA: the warps' FP64 chains spread over the SMs' sub-partitions
       if ((st = taps_allow_dyn_smem((const void*)fd_bisect_kernel, maxsm_optin)) != TAPS_OK) break;
       fd_bisect_kernel<<<(unsigned)((32LL * n + 63) / 64), 64, sizeof(double) * 2 * n, s>>>(T->dd, T->ee, n, lam);
-      // eigenvectors in shared memory where IV_COLS of them fit (n <= ~670), else one thread per
-      // eigenvector on global arrays, in 32-thread CTAs: the chains spread over the SMs
-      if (iv_smem(n) + 1024 <= (size_t)maxsm_optin) {
-        if ((st = taps_allow_dyn_smem((const void*)fd_invit_smem_kernel, maxsm_optin)) != TAPS_OK) break;
-        fd_invit_smem_kernel<<<(n + IV_COLS - 1) / IV_COLS, 32, iv_smem(n), s>>>(T->dd, T->ee, lam, n, A);
-      } else {
+      // eigenvectors in shared memory, as many to a CTA as fit, else one thread per eigenvector
+      // on global arrays, in 32-thread CTAs: the chains spread over the SMs
+      int cols = 8;
+      while (cols > 0 && iv_smem(n, cols) + 1024 > (size_t)maxsm_optin) cols >>= 1;
+      if (cols == 8) st = iv_launch<8>(T->dd, T->ee, lam, n, A, maxsm_optin, s);
+      else if (cols == 4) st = iv_launch<4>(T->dd, T->ee, lam, n, A, maxsm_optin, s);
+      else if (cols == 2) st = iv_launch<2>(T->dd, T->ee, lam, n, A, maxsm_optin, s);
+      else if (cols == 1) st = iv_launch<1>(T->dd, T->ee, lam, n, A, maxsm_optin, s);
+      if (st != TAPS_OK) break;
+      if (cols == 0) {
         fd_invit_kernel<<<(n + 31) / 32, 32, 0, s>>>(T->dd, T->ee, lam, n, A, W);
       }
       // symmetric orthogonalisation: E in W, the corrected vectors back into A
