@@ -474,47 +474,17 @@ extern "C" int taps_profile_get(taps_problem* P, int cls, long long* launches, d
 // Problem
 // ---------------------------------------------------------------------------------
 static void free_ws(taps_problem* P) {
-  for (int d = 0; d < TAPS_MAX_DIMS; ++d) {
-    cudaFree(P->d_gram[d]);
-    cudaFree(P->d_h[d]);
-    P->d_gram[d] = P->d_h[d] = nullptr;
-  }
-  for (int d = 0; d < TAPS_MAX_DIMS; ++d) {
-    cudaFree(P->d_Usnap[d]);
-    P->d_Usnap[d] = nullptr;
-  }
   loop_destroy(P);
-  cudaFree(P->d_C);
-  cudaFree(P->d_c);
-  cudaFree(P->d_Call);
-  cudaFree(P->d_call);
-  cudaFree(P->d_ticket);
-  P->d_Call = P->d_call = nullptr;
-  P->d_ticket = nullptr;
-  cudaFree(P->d_F);
-  cudaFree(P->d_blocks);
-  cudaFree(P->d_lu);
-  cudaFree(P->d_Y);
-  cudaFree(P->d_Uold);
-  cudaFree(P->d_ts);
-  P->d_ts = nullptr;
-  cudaFree(P->d_md);
-  P->d_md = nullptr;
-  cudaFree(P->d_fdw);
-  P->d_fdw = nullptr;
-  cudaFree(P->d_partial);
-  cudaFree(P->d_scal);
-  cudaFree(P->d_bigG);
-  cudaFree(P->d_Yres);
-  P->d_Yres = nullptr;
-  cudaFree(P->d_ticket_all);
-  P->d_ticket_all = nullptr;
+  cudaFree(P->d_ws);
   if (P->h_scal) cudaFreeHost(P->h_scal);
-  if (P->h_part) cudaFreeHost(P->h_part);
-  P->h_part = nullptr;
   graph_destroy(P);
-  P->d_C = P->d_c = P->d_F = P->d_blocks = P->d_lu = P->d_Y = P->d_Uold = nullptr;
-  P->d_partial = P->d_scal = P->d_bigG = P->h_scal = nullptr;
+  for (int d = 0; d < TAPS_MAX_DIMS; ++d) P->d_gram[d] = P->d_h[d] = P->d_Usnap[d] = nullptr;
+  P->d_ws = nullptr;
+  P->d_ticket = P->d_ticket_all = nullptr;
+  P->d_C = P->d_c = P->d_Call = P->d_call = P->d_F = P->d_blocks = P->d_lu = P->d_Y = P->d_Uold = nullptr;
+  P->d_ts = P->d_md = P->d_fdw = nullptr;
+  P->d_partial = P->d_scal = P->d_bigG = P->d_Yres = nullptr;
+  P->h_scal = P->h_part = nullptr;
   P->ws_M = 0;
 }
 
@@ -545,11 +515,24 @@ extern "C" void taps_problem_destroy(taps_problem* P) {
   delete P;
 }
 
+// One device allocation and one pinned one hold every part: some thirty allocations and frees, and
+// a pinned mirror as long as the Gram partials where only residual sums go through it, were
+// 0.7 of the 7.8 ms of a set-up and solve of the space-parameter problem.
 int taps_ws_ensure(taps_problem* P, int M) {
   if (M <= P->ws_M) return TAPS_OK;
   if (P->stream) TAPS_CUDA(cudaStreamSynchronize(P->stream));
   free_ws(P);
   P->c0_valid = 0;
+  struct Part {
+    void** p;
+    size_t off;
+  };
+  std::vector<Part> parts;
+  size_t total = 0;
+  auto want = [&](void* p, size_t bytes) {   // p: address of the pointer
+    parts.push_back({(void**)p, total});
+    total += std::max<size_t>((bytes + 255) / 256 * 256, 256);
+  };
   int nbmax = 0, D = P->D;
   size_t part = 0, bigG = 0, yres = 0, part_all = 0, ts = 0;
   for (int d = 0; d < D; ++d) {
@@ -557,9 +540,9 @@ int taps_ws_ensure(taps_problem* P, int M) {
     int nops = P->tt.nops[d];
     nbmax = std::max(nbmax, dm->nb);
     ts = std::max(ts, taps_ts_scratch_doubles(dm->hb, std::min(M, 64)));
-    TAPS_TRY(taps_alloc((void**)&P->d_gram[d], sizeof(double) * nops * M * M));
-    TAPS_TRY(taps_alloc((void**)&P->d_h[d], sizeof(double) * P->Rf * M));
-    TAPS_TRY(taps_alloc((void**)&P->d_Usnap[d], sizeof(double) * dm->nf * M));
+    want(&P->d_gram[d], sizeof(double) * nops * M * M);
+    want(&P->d_h[d], sizeof(double) * P->Rf * M);
+    want(&P->d_Usnap[d], sizeof(double) * dm->nf * M);
     size_t gp = (size_t)((dm->nf + 7) / 8) * (nops * M * M + P->Rf * M);
     part = std::max(part, gp);
     part_all += gp;
@@ -577,29 +560,32 @@ int taps_ws_ensure(taps_problem* P, int M) {
   size_t MM = (size_t)M * M;
   int nfm = P->nf_max;
   const size_t cs = (size_t)P->tt.cs;   // TAPS_NUM_OPS unless weighted operators add slots
-  TAPS_TRY(taps_alloc((void**)&P->d_C, sizeof(double) * cs * MM));
-  TAPS_TRY(taps_alloc((void**)&P->d_c, sizeof(double) * P->Rf * M));
-  TAPS_TRY(taps_alloc((void**)&P->d_Call, sizeof(double) * D * cs * MM));
-  TAPS_TRY(taps_alloc((void**)&P->d_call, sizeof(double) * D * P->Rf * M));
-  TAPS_TRY(taps_alloc((void**)&P->d_ticket, sizeof(unsigned) * 64));   // >= M / 8 + 1
+  want(&P->d_C, sizeof(double) * cs * MM);
+  want(&P->d_c, sizeof(double) * P->Rf * M);
+  want(&P->d_Call, sizeof(double) * D * cs * MM);
+  want(&P->d_call, sizeof(double) * D * P->Rf * M);
+  want(&P->d_ticket, sizeof(unsigned) * 64);   // >= M / 8 + 1
+  want(&P->d_ticket_all, sizeof(unsigned) * 32 * TAPS_MAX_DIMS);
+  want(&P->d_F, sizeof(double) * nfm * M);
+  want(&P->d_blocks, sizeof(double) * nfm * nbmax * MM);
+  want(&P->d_lu, sizeof(double) * MM);
+  want(&P->d_Y, sizeof(double) * cs * nfm * M);
+  want(&P->d_Uold, sizeof(double) * nfm * M);
+  want(&P->d_ts, sizeof(double) * ts);
+  want(&P->d_fdw, sizeof(double) * taps_fdw_scratch_doubles(nfm, M));
+  want(&P->d_md, sizeof(double) * taps_md_scratch_doubles(nfm, M, P->Rf));
+  want(&P->d_partial, sizeof(double) * part);
+  want(&P->d_scal, sizeof(double) * 2 * M * D + 64);
+  want(&P->d_bigG, sizeof(double) * bigG);
+  want(&P->d_Yres, sizeof(double) * yres);
+  TAPS_TRY(taps_alloc(&P->d_ws, total));
+  for (const Part& w : parts) *w.p = (char*)P->d_ws + w.off;
   TAPS_CUDA(cudaMemsetAsync(P->d_ticket, 0, sizeof(unsigned) * 64, P->stream));
-  TAPS_TRY(taps_alloc((void**)&P->d_ticket_all, sizeof(unsigned) * 32 * TAPS_MAX_DIMS));
   TAPS_CUDA(cudaMemsetAsync(P->d_ticket_all, 0, sizeof(unsigned) * 32 * TAPS_MAX_DIMS, P->stream));
-  TAPS_TRY(taps_alloc((void**)&P->d_F, sizeof(double) * nfm * M));
-  TAPS_TRY(taps_alloc((void**)&P->d_blocks, sizeof(double) * nfm * nbmax * MM));
-  TAPS_TRY(taps_alloc((void**)&P->d_lu, sizeof(double) * MM));
-  TAPS_TRY(taps_alloc((void**)&P->d_Y, sizeof(double) * cs * nfm * M));
-  TAPS_TRY(taps_alloc((void**)&P->d_Uold, sizeof(double) * nfm * M));
-  TAPS_TRY(taps_alloc((void**)&P->d_ts, sizeof(double) * ts));
-  TAPS_TRY(taps_alloc((void**)&P->d_fdw, sizeof(double) * taps_fdw_scratch_doubles(nfm, M)));
-  TAPS_TRY(taps_alloc((void**)&P->d_md, sizeof(double) * taps_md_scratch_doubles(nfm, M, P->Rf)));
   TAPS_CUDA(cudaMemsetAsync(P->d_md, 0, sizeof(double) * taps_md_scratch_doubles(nfm, M, P->Rf), P->stream));
-  TAPS_TRY(taps_alloc((void**)&P->d_partial, sizeof(double) * part));
-  TAPS_TRY(taps_alloc((void**)&P->d_scal, sizeof(double) * 2 * M * D + 64));
-  TAPS_TRY(taps_alloc((void**)&P->d_bigG, sizeof(double) * bigG));
-  TAPS_TRY(taps_alloc((void**)&P->d_Yres, sizeof(double) * yres));
-  TAPS_CUDA(cudaMallocHost((void**)&P->h_scal, sizeof(double) * (2 * M * D + 64)));
-  TAPS_CUDA(cudaMallocHost((void**)&P->h_part, sizeof(double) * part));
+  const size_t hs = 2 * (size_t)M * D + 64;
+  TAPS_CUDA(cudaMallocHost((void**)&P->h_scal, sizeof(double) * (hs + std::max(als_part, (size_t)3 * 64))));
+  P->h_part = P->h_scal + hs;
   P->partial_len = part;
   P->bigG_len = bigG;
   P->ws_M = M;

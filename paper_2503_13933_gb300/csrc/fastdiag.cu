@@ -720,10 +720,10 @@ __global__ void fd_invit_kernel(const double* __restrict__ d, const double* __re
 }
 
 // The same with T, the factors and the iterate in shared memory: IV_COLS eigenvectors to a CTA
-// of one warp, as many of 8, 4, 2, 1 as fit (n <= ~820, 1560, 2820, 4770).  The passes are chains over the nodes whose global-memory arrays, written and
-// read back by the same thread, were most of their time (254 nodes: 1055 us;
-// 1534 nodes, 4 to a CTA: 157 ms on global arrays, 95 ms here, 11.5 ms with
-// the narrower clusters).
+// of one warp, as many of 8, 4, 2, 1 as fit (n <= ~820, 1560, 2820, 4720).  The passes are chains
+// over the nodes whose global-memory arrays, written and read back by the same thread, were most
+// of their time (254 nodes: 1055 and 644 us; 1532 nodes, 4 to a CTA: 157 and 95 ms, 11.5 with the
+// narrower clusters).
 static size_t iv_smem(int n, int cols) {
   return sizeof(double) * (2 * (size_t)n + 4 * (size_t)n * cols) + (size_t)n * cols;
 }
@@ -1470,14 +1470,6 @@ int taps_fd_eligible(const taps_problem* P, int d, int* slotA, int* slotB) {
 
 static void fd_pending_free(FdPending& T) {
   cudaFree(T.A);
-  cudaFree(T.B);
-  cudaFree(T.V);
-  cudaFree(T.tmp);
-  cudaFree(T.bt);
-  cudaFree(T.dd);
-  cudaFree(T.ee);
-  cudaFree(T.lam);
-  cudaFree(T.W);
   memset(&T, 0, sizeof(T));
 }
 
@@ -1674,16 +1666,21 @@ static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, FdEntry**
     if ((st = taps_alloc((void**)&E.Phi, sizeof(double) * nn)) != TAPS_OK) break;
     if ((st = taps_alloc((void**)&E.PhiT, sizeof(double) * nn)) != TAPS_OK) break;
     if ((st = taps_alloc((void**)&E.mu, sizeof(double) * n)) != TAPS_OK) break;
-    if ((st = taps_alloc((void**)&T->A, sizeof(double) * nn)) != TAPS_OK) break;
-    if ((st = taps_alloc((void**)&T->B, sizeof(double) * nn)) != TAPS_OK) break;
-    if ((st = taps_alloc((void**)&T->V, sizeof(double) * nn)) != TAPS_OK) break;
-    if ((st = taps_alloc((void**)&T->tmp, sizeof(double) * 2 * n)) != TAPS_OK) break;
-    if ((st = taps_alloc((void**)&T->bt, sizeof(double) * n)) != TAPS_OK) break;
-    if ((st = taps_alloc((void**)&T->dd, sizeof(double) * n)) != TAPS_OK) break;
-    if ((st = taps_alloc((void**)&T->ee, sizeof(double) * n)) != TAPS_OK) break;
-    if (hasA) {
-      if ((st = taps_alloc((void**)&T->lam, sizeof(double) * n)) != TAPS_OK) break;
-      if ((st = taps_alloc((void**)&T->W, sizeof(double) * 5 * nn)) != TAPS_OK) break;
+    // eigenvectors to a CTA of the inverse iteration: as many as fit its shared memory, 0 for the
+    // kernel on global arrays
+    int cols = 8;
+    while (cols > 0 && iv_smem(n, cols) + 1024 > (size_t)maxsm_optin) cols >>= 1;
+    {
+      const size_t nW = hasA ? (cols == 0 ? 5 : 2) * nn : 0;
+      if ((st = taps_alloc((void**)&T->A, sizeof(double) * (3 * nn + nW + 6 * (size_t)n))) != TAPS_OK) break;
+      T->B = T->A + nn;
+      T->V = T->B + nn;
+      T->tmp = T->V + nn;
+      T->bt = T->tmp + 2 * n;
+      T->dd = T->bt + n;
+      T->ee = T->dd + n;
+      T->lam = T->ee + n;
+      T->W = T->lam + n;
     }
     double *A = T->A, *B = T->B, *V = T->V, *W = T->W, *lam = T->lam;
     const size_t bsz = (size_t)n * dm->nb;
@@ -1709,8 +1706,6 @@ static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, FdEntry**
       fd_bisect_kernel<<<(unsigned)((32LL * n + 63) / 64), 64, sizeof(double) * 2 * n, s>>>(T->dd, T->ee, n, lam);
       // eigenvectors in shared memory, as many to a CTA as fit, else one thread per eigenvector
       // on global arrays, in 32-thread CTAs: the chains spread over the SMs
-      int cols = 8;
-      while (cols > 0 && iv_smem(n, cols) + 1024 > (size_t)maxsm_optin) cols >>= 1;
       if (cols == 8) st = iv_launch<8>(T->dd, T->ee, lam, n, A, maxsm_optin, s);
       else if (cols == 4) st = iv_launch<4>(T->dd, T->ee, lam, n, A, maxsm_optin, s);
       else if (cols == 2) st = iv_launch<2>(T->dd, T->ee, lam, n, A, maxsm_optin, s);

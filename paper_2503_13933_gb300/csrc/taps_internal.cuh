@@ -129,8 +129,10 @@ struct taps_problem {
   double* d_pq[TAPS_MAX_DIMS];           // [Rf][nf_d] Phi_d^T q_r (fast diagonalisation)
   double* d_beta;                        // [Rf] source amplitudes
   double* d_opband[TAPS_MAX_DIMS];       // [nops_d][nf_d][nb] bands of the distinct ops
-  // Workspace, grown to the largest mode count seen (ws_M).
+  // Workspace, grown to the largest mode count seen (ws_M): parts of d_ws, and of one pinned
+  // allocation at h_scal.
   int ws_M;
+  void* d_ws;
   double* d_gram[TAPS_MAX_DIMS];  // [nops_d][M][M]
   double* d_h[TAPS_MAX_DIMS];     // [Rf][M]
   double* d_C;        // [tt.cs][M][M] coefficient matrices of the current dim
@@ -420,7 +422,7 @@ int taps_fd_prepare_all(taps_problem* P, int solver, int M);
 struct FdPending {
   FdEntry* E;
   taps_problem* P;
-  double *A, *B, *V, *tmp, *bt, *dd, *ee, *lam, *W;
+  double *A, *B, *V, *tmp, *bt, *dd, *ee, *lam, *W;   // parts of one allocation at A
 };
 // Mode-side diagonalisation (modediag.cu): eligibility of dim d at M modes (slots of
 // the mass-like operator X and the other Y), scratch size, and the solve.
