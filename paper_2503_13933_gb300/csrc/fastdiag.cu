@@ -1413,8 +1413,10 @@ __global__ void __launch_bounds__(128) fd_small_solve_quad_kernel(const double* 
 // One CTA per node i (M > 32): solve (mu_i C_A + C_B) y = g_i by LU with partial pivoting in
 // shared memory (small_lu.cuh).  A zero or non-finite pivot is reported as
 // TAPS_DEV_SINGULAR.  1534 systems of 100 modes: 1.97 ms with the pivot search between two
-// barriers of a step, 1.32 ms now (0.85 ms of FP64 issue).
-#define FS_THREADS 256
+// barriers of a step, 1.30 ms now (0.85 ms of FP64 issue).  Eleven update warps beside the pivot's
+// load the four sub-partitions more evenly than seven (1.35 ms; 183 and 156 us for 16 systems);
+// fifteen take 1.31 ms.
+#define FS_THREADS 384
 __global__ void __launch_bounds__(FS_THREADS, 2) fd_small_solve_kernel(const double* __restrict__ CA,
                                                                        const double* __restrict__ CB,
                                                                        const double* __restrict__ mu,
