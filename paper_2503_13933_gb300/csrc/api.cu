@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <type_traits>
 #include <vector>
 
 #include "taps_internal.cuh"
@@ -1190,23 +1191,37 @@ extern "C" int taps_solve(taps_problem* P, taps_factors* U, const taps_solve_opt
 // eval_factor_kernel; eval_gemm_kernel streams the output with register tiles.
 // ---------------------------------------------------------------------------------
 
+// The factor rows of every dim in one launch, a thread per entry of G (one launch per dim was most
+// of a small grid's time).
+struct GatherDims {
+  const double* U[TAPS_MAX_DIMS];
+  int nf[TAPS_MAX_DIMS], off[TAPS_MAX_DIMS], start[TAPS_MAX_DIMS], step[TAPS_MAX_DIMS];
+};
+
 template <typename T>
-__global__ void gather_rows_kernel(const double* U, int nf, int off, int start, int step, int count,
-                                   int M, T* G) {
-  int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= count * M) return;
-  int j = idx / M, m = idx % M;
-  int node = start + step * j;
-  int fj = node - off;
-  G[idx] = (fj >= 0 && fj < nf) ? (T)U[(size_t)m * nf + fj] : (T)0;
+__global__ void gather_rows_kernel(GatherDims gd, GridSpec gs, int M, long long total, T* G) {
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= total) return;
+  int d = 0;
+  while (d + 1 < gs.D && idx >= gs.goff[d + 1]) ++d;
+  const int loc = (int)(idx - gs.goff[d]);
+  const int j = loc / M, m = loc % M;
+  const int node = gd.start[d] + gd.step[d] * j;
+  const int fj = node - gd.off[d];
+  G[idx] = (fj >= 0 && fj < gd.nf[d]) ? (T)gd.U[d][(size_t)m * gd.nf[d] + fj] : (T)0;
 }
 
-// X[x][m] = prod_{d in [d0, d1)} G_d[i_d(x)][m], x in C order over dims d0..d1-1.
+// X[x][m] = prod_{d in [d0, d1)} G_d[i_d(x)][m], x in C order over dims d0..d1-1: A over the
+// leading dims (the first nA entries), then B over the others.
 template <typename T>
-__global__ void eval_factor_kernel(const T* __restrict__ G, GridSpec gs, int d0, int d1, int M,
-                                   long long nx, T* __restrict__ X) {
+__global__ void eval_factor_kernel(const T* __restrict__ G, GridSpec gs, int split, int M, long long nA,
+                                   long long nB, T* __restrict__ A, T* __restrict__ B) {
   long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= nx * M) return;
+  if (idx >= nA + nB) return;
+  const bool first = idx < nA;
+  const int d0 = first ? 0 : split, d1 = first ? split : gs.D;
+  T* __restrict__ X = first ? A : B;
+  if (!first) idx -= nA;
   long long x = idx / M;
   int m = (int)(idx - x * M);
   T v = (T)1;
@@ -1219,7 +1234,7 @@ __global__ void eval_factor_kernel(const T* __restrict__ G, GridSpec gs, int d0,
   X[idx] = v;
 }
 
-// out[r][c] = sum_m A[r][m] B[c][m].  CTA tile 128 x 128 (256 threads), thread tile
+// out[r][c] = sum_m A[r][m] B[c][m], FP32.  CTA tile 128 x 128 (256 threads), thread tile
 // 8 x 8 with rows ty + 16a and columns tx + 16b, so that shared-memory reads are
 // broadcasts / conflict-free and every warp store covers two 64-byte row segments.
 // The tiles are stored transposed ([m][row]) with a padded stride (129) so that the
@@ -1236,13 +1251,12 @@ __device__ __forceinline__ void unpack2(unsigned long long v, float& a, float& b
   asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
 }
 
-template <typename T>
-__device__ __forceinline__ void eval_fill(const T* __restrict__ A, const T* __restrict__ B, long long r0,
-                                          int c0, int nr, int nc, int M, T* As, T* Bs) {
+__device__ __forceinline__ void eval_fill(const float* __restrict__ A, const float* __restrict__ B, long long r0,
+                                          int c0, int nr, int nc, int M, float* As, float* Bs) {
   for (int idx = threadIdx.x; idx < EB * M; idx += blockDim.x) {
     int r = idx / M, m = idx - r * M;
-    As[m * EBP + r] = (r < nr) ? A[(r0 + r) * M + m] : (T)0;
-    Bs[m * EBP + r] = (r < nc) ? B[(long long)(c0 + r) * M + m] : (T)0;
+    As[m * EBP + r] = (r < nr) ? A[(r0 + r) * M + m] : 0.0f;
+    Bs[m * EBP + r] = (r < nc) ? B[(long long)(c0 + r) * M + m] : 0.0f;
   }
 }
 
@@ -1256,7 +1270,7 @@ __global__ void __launch_bounds__(256) eval_gemm_f32_kernel(const float* __restr
   const int c0 = blockIdx.y * EB;
   const int nr = (int)min((long long)EB, R - r0);
   const int nc = min(EB, C - c0);
-  eval_fill<float>(A, B, r0, c0, nr, nc, M, As, Bs);
+  eval_fill(A, B, r0, c0, nr, nc, M, As, Bs);
   __syncthreads();
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
   unsigned long long acc[8][4];
@@ -1293,45 +1307,75 @@ __global__ void __launch_bounds__(256) eval_gemm_f32_kernel(const float* __restr
   }
 }
 
-__global__ void __launch_bounds__(256) eval_gemm_f64_kernel(const double* __restrict__ A,
+// The FP64 product: CTA tile 64 x 128, thread tile 4 x 8.  FP64 issue is the bound (M FMAs per
+// value against 8 bytes written), so what counts is how evenly the SMs are loaded: half the rows
+// of the FP32 tile leave a shorter last wave, and groups of 16 rows or columns outside the grid
+// are not multiplied.  The modes go through shared memory ED_MODES at a time, so that two CTAs fit
+// an SM whatever M is and one's loads hide behind the other's products.  With 128 x 128 tiles
+// multiplied in full and all modes at once, and now: 347 and 337 us for 10201 x 1111 values of 17
+// modes, 760 and 739 us for 4900 x 770 of 90, 131 and 72 us for 400 x 1620 of 30.
+#define ED_ROWS 64
+#define ED_MODES 32
+static size_t eval_f64_smem(int M) {
+  return (size_t)std::min(M, ED_MODES) * (ED_ROWS + 1 + EBP) * sizeof(double);
+}
+
+__global__ void __launch_bounds__(256, 2) eval_gemm_f64_kernel(const double* __restrict__ A,
                                                             const double* __restrict__ B, long long R,
                                                             int C, int M, double* __restrict__ out) {
   extern __shared__ __align__(16) double smd[];
-  double* As = smd;
-  double* Bs = smd + M * EBP;
-  const long long r0 = (long long)blockIdx.x * EB;
+  double* As = smd;                                        // [min(M, ED_MODES)][ED_ROWS + 1]
+  double* Bs = smd + min(M, ED_MODES) * (ED_ROWS + 1);     // [min(M, ED_MODES)][EBP]
+  const long long r0 = (long long)blockIdx.x * ED_ROWS;
   const int c0 = blockIdx.y * EB;
-  const int nr = (int)min((long long)EB, R - r0);
+  const int nr = (int)min((long long)ED_ROWS, R - r0);
   const int nc = min(EB, C - c0);
-  eval_fill<double>(A, B, r0, c0, nr, nc, M, As, Bs);
-  __syncthreads();
   const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-  for (int half = 0; half < 2; ++half) {  // 4 of the 8 rows per pass keeps registers bounded
-    double acc[4][8];
+  const int na = (nr + 15) >> 4, nb = (nc + 15) >> 4;   // groups of 16 inside the grid
+  double acc[4][8];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int b = 0; b < 8; ++b) acc[a][b] = 0.0;
-    for (int m = 0; m < M; ++m) {
+    for (int b = 0; b < 8; ++b) acc[a][b] = 0.0;
+  auto multiply = [&](auto full, int mc) {
+    for (int m = 0; m < mc; ++m) {
       double av[4], bv[8];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = As[m * EBP + ty + 16 * (4 * half + a)];
+      for (int a = 0; a < 4; ++a) av[a] = As[m * (ED_ROWS + 1) + ty + 16 * a];
 #pragma unroll
       for (int b = 0; b < 8; ++b) bv[b] = Bs[m * EBP + tx + 16 * b];
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+      for (int b = 0; b < 8; ++b) {
+        if (!decltype(full)::value && b >= nb) break;
 #pragma unroll
-        for (int b = 0; b < 8; ++b) acc[a][b] += av[a] * bv[b];
+        for (int a = 0; a < 4; ++a)
+          if (decltype(full)::value || a < na) acc[a][b] += av[a] * bv[b];
+      }
     }
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      int r = ty + 16 * (4 * half + a);
-      if (r >= nr) continue;
-      double* o = out + (r0 + r) * (long long)C + c0 + tx;
-#pragma unroll
-      for (int b = 0; b < 8; ++b)
-        if (tx + 16 * b < nc) o[16 * b] = acc[a][b];
+  };
+  for (int m0 = 0; m0 < M; m0 += ED_MODES) {
+    const int mc = min(ED_MODES, M - m0);
+    if (m0 > 0) __syncthreads();
+    for (int idx = threadIdx.x; idx < ED_ROWS * mc; idx += blockDim.x) {
+      const int r = idx / mc, m = idx - r * mc;
+      As[m * (ED_ROWS + 1) + r] = (r < nr) ? A[(r0 + r) * M + m0 + m] : 0.0;
     }
+    for (int idx = threadIdx.x; idx < EB * mc; idx += blockDim.x) {
+      const int r = idx / mc, m = idx - r * mc;
+      Bs[m * EBP + r] = (r < nc) ? B[(long long)(c0 + r) * M + m0 + m] : 0.0;
+    }
+    __syncthreads();
+    if (na == 4 && nb == 8) multiply(std::true_type{}, mc);
+    else multiply(std::false_type{}, mc);
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int r = ty + 16 * a;
+    if (r >= nr) continue;
+    double* o = out + (r0 + r) * (long long)C + c0 + tx;
+#pragma unroll
+    for (int b = 0; b < 8; ++b)
+      if (tx + 16 * b < nc) o[16 * b] = acc[a][b];
   }
 }
 
@@ -1388,37 +1432,37 @@ extern "C" int taps_eval_grid(const taps_problem* Pc, const taps_factors* U, con
     P->eval_attr_set = 1;
   }
   int tk = prof_begin(P, TAPS_PROF_EVAL);
+  GatherDims gd;
+  memset(&gd, 0, sizeof(gd));
   for (int d = 0; d < P->D; ++d) {
-    const taps_dim* dm = P->dims[d];
-    int n = count[d] * M;
-    if (out_dtype == TAPS_FP64)
-      gather_rows_kernel<double><<<(n + 255) / 256, 256, 0, s>>>(U->d_U[d], dm->nf, dm->off, start[d],
-                                                                 step[d], count[d], M,
-                                                                 (double*)G + gs.goff[d]);
-    else
-      gather_rows_kernel<float><<<(n + 255) / 256, 256, 0, s>>>(U->d_U[d], dm->nf, dm->off, start[d],
-                                                                step[d], count[d], M,
-                                                                (float*)G + gs.goff[d]);
+    gd.U[d] = U->d_U[d];
+    gd.nf[d] = P->dims[d]->nf;
+    gd.off[d] = P->dims[d]->off;
+    gd.start[d] = start[d];
+    gd.step[d] = step[d];
   }
+  const unsigned gg = (unsigned)((goff + 255) / 256);
+  if (out_dtype == TAPS_FP64) gather_rows_kernel<double><<<gg, 256, 0, s>>>(gd, gs, M, goff, (double*)G);
+  else gather_rows_kernel<float><<<gg, 256, 0, s>>>(gd, gs, M, goff, (float*)G);
+  const long long nA = rows * M, nB = cols * M;
+  const unsigned fg = (unsigned)((nA + nB + 255) / 256);
   if (use_tc) {
     st = taps_eval_tc(P, (const float*)G, gs, split, M, rows, cols, (char*)G + gbytes, (float*)out_dev);
     if (st != TAPS_OK) return st;
   } else if (out_dtype == TAPS_FP64) {
     double* A = (double*)G + goff;
     double* B = A + rows * M;
-    eval_factor_kernel<double><<<(unsigned)((rows * M + 255) / 256), 256, 0, s>>>((const double*)G, gs, 0, split, M, rows, A);
-    eval_factor_kernel<double><<<(unsigned)((cols * M + 255) / 256), 256, 0, s>>>((const double*)G, gs, split, P->D, M, cols, B);
-    dim3 eg((unsigned)((rows + EB - 1) / EB), (unsigned)((cols + EB - 1) / EB));
-    eval_gemm_f64_kernel<<<eg, 256, (size_t)M * 2 * EBP * sizeof(double), s>>>(A, B, rows, (int)cols, M, (double*)out_dev);
+    eval_factor_kernel<double><<<fg, 256, 0, s>>>((const double*)G, gs, split, M, nA, nB, A, B);
+    dim3 eg((unsigned)((rows + ED_ROWS - 1) / ED_ROWS), (unsigned)((cols + EB - 1) / EB));
+    eval_gemm_f64_kernel<<<eg, 256, eval_f64_smem(M), s>>>(A, B, rows, (int)cols, M, (double*)out_dev);
   } else {
     float* A = (float*)G + goff;
     float* B = A + rows * M;
-    eval_factor_kernel<float><<<(unsigned)((rows * M + 255) / 256), 256, 0, s>>>((const float*)G, gs, 0, split, M, rows, A);
-    eval_factor_kernel<float><<<(unsigned)((cols * M + 255) / 256), 256, 0, s>>>((const float*)G, gs, split, P->D, M, cols, B);
+    eval_factor_kernel<float><<<fg, 256, 0, s>>>((const float*)G, gs, split, M, nA, nB, A, B);
     dim3 eg((unsigned)((rows + EB - 1) / EB), (unsigned)((cols + EB - 1) / EB));
     eval_gemm_f32_kernel<<<eg, 256, (size_t)M * 2 * EBP * sizeof(float), s>>>(A, B, rows, (int)cols, M, (float*)out_dev);
   }
-  P->prof->launches[TAPS_PROF_EVAL] += P->D + 2;  // gathers, two factor products / images, product
+  P->prof->launches[TAPS_PROF_EVAL] += use_tc ? 3 : 2;  // beside the product: the gather, and the factor products or two images
   prof_end(P, TAPS_PROF_EVAL, tk, 2.0 * M * (double)total + (double)(rows + cols) * M * (P->D - 1),
            (double)esz * total);
   cudaError_t e = cudaGetLastError();
