@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(TDS_THREADS)
   }
   cluster.sync();
   for (int k = 0; k + 2 < n; ++k) {
-    const int len = n - k - 1, nact = (len + 31) / 32;   // warps with entries of the column
+    const int len = n - k - 1, nact = min((len + 31) / 32, nwarps);   // warps with entries of the column
     // column k below the diagonal, from the owners of its rows
     if (warp < nact) {
       double s2 = 0.0;
