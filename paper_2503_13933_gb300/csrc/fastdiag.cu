@@ -1542,16 +1542,19 @@ static bool td_grid_ok(size_t smem, int maxsm) {
 // TD_CLUSTER_MOST nodes, where its cheaper barriers win, then in the shared memory of all num_sms
 // SMs while its rows fit (152: n <= ~1820), else in global memory.  Cluster and chip: 1.75 and
 // 2.34 ms for 254 nodes, 3.55 and 3.69 for 382, 6.28 and 5.21 for 510, 10.4 and 6.78 for 638.
+// beside: a batch enqueues many instances' decompositions at once, and nine clusters side by side
+// do more of them than one chip-wide kernel after another (24 instances of three dims of 460 to
+// 640 nodes: 303 and 540 ms; of 700 to 1024: 1.05 and 1.20 s).
 // xch: 4 n doubles and two words of workspace.
 #define TD_CLUSTER_MOST 448
 static int td_run(double* A, double* V, double* tmp, double* bt, double* dd, double* ee, int n, int maxsm,
-                  int num_sms, double* xch, int* status, cudaStream_t s) {
+                  int num_sms, bool beside, double* xch, int* status, cudaStream_t s) {
   const size_t dsm16 = sizeof(double) * ((size_t)((n + 15) / 16) * n + 3 * (size_t)n);
   const size_t dsm8 = sizeof(double) * ((size_t)((n + 7) / 8) * n + 3 * (size_t)n);
   const size_t gsm = sizeof(double) * 3 * (size_t)n;
   const size_t grd = sizeof(double) * ((size_t)((n + num_sms - 1) / num_sms) * n + 3 * (size_t)n);
   cudaError_t ce;
-  const bool small = n <= TD_CLUSTER_MOST || grd + 1024 > (size_t)maxsm || n > TDG_THREADS * TDG_PER;
+  const bool small = beside || n <= TD_CLUSTER_MOST || grd + 1024 > (size_t)maxsm || n > TDG_THREADS * TDG_PER;
   if (small && dsm16 + 1024 <= (size_t)maxsm && td_cluster_ok<16>((const void*)fd_tridiag_dsmem_kernel<16>, dsm16, TDS_THREADS)) {
     ce = td_launch<16>(fd_tridiag_dsmem_kernel<16>, TDS_THREADS, dsm16, s, (const double*)A, V, bt, dd, ee, n);
   } else if (small && dsm8 + 1024 <= (size_t)maxsm && td_cluster_ok<8>((const void*)fd_tridiag_dsmem_kernel<8>, dsm8, TDS_THREADS)) {
@@ -1635,7 +1638,7 @@ static int iv_launch(const double* dd, const double* ee, const double* lam, int 
 // waiting for it: the entry is registered at once (pending, with an event recorded
 // after its last kernel) and the temporaries are returned in *T for fd_finish.  An
 // entry that already exists, pending on another stream, makes P's stream wait for it.
-static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, FdEntry** out, FdPending* T) {
+static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, bool beside, FdEntry** out, FdPending* T) {
   memset(T, 0, sizeof(*T));
   for (int k = 0; k < dm->nfd; ++k)
     if (dm->fd[k].opA == opA && dm->fd[k].opB == opB) {
@@ -1700,7 +1703,7 @@ static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, FdEntry**
       if ((st = fd_lsolve(B, linv, V, n, dm->hb, 1, W, s)) != TAPS_OK) break;
       fd_symmetrize_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(W, n, A);
       if (cudaMemsetAsync(V, 0, sizeof(double) * nn, s) != cudaSuccess) { st = TAPS_ERR_CUDA; break; }
-      if ((st = td_run(A, V, T->tmp, T->bt, T->dd, T->ee, n, maxsm_optin, P->num_sms, W, P->d_status, s)) != TAPS_OK) break;
+      if ((st = td_run(A, V, T->tmp, T->bt, T->dd, T->ee, n, maxsm_optin, P->num_sms, beside, W, P->d_status, s)) != TAPS_OK) break;
       // eigenvalues (warp each), eigenvectors (thread each), back-transform (warp each),
       // all into A, which the tridiagonalisation no longer needs
       // two warps per CTA: the warps' FP64 chains spread over the SMs' sub-partitions
@@ -1772,7 +1775,7 @@ static int fd_finish(FdPending& T) {
 static int fd_prepare(taps_problem* P, int d, taps_dim* dm, int opA, int opB, FdEntry** out) {
   (void)d;
   FdPending T;
-  int st = fd_enqueue(P, dm, opA, opB, out, &T);
+  int st = fd_enqueue(P, dm, opA, opB, false, out, &T);
   if (st != TAPS_OK) return st;
   return fd_finish(T);
 }
@@ -1853,7 +1856,7 @@ int taps_fd_to_nodal(taps_problem* P, const FdEntry* E, const double* Y, int n, 
 // their temporaries in *pend; the finish half waits, checks and frees.  Batches
 // enqueue many problems (each on its own stream) before finishing any, so the
 // decompositions of different instances run concurrently.
-int taps_fd_prepare_enqueue(taps_problem* P, int solver, int M, std::vector<FdPending>* pend) {
+int taps_fd_prepare_enqueue(taps_problem* P, int solver, int M, bool beside, std::vector<FdPending>* pend) {
   if (solver != TAPS_SOLVER_FASTDIAG && solver != TAPS_SOLVER_MODEDIAG) return TAPS_OK;
   for (int d = 0; d < P->D; ++d) {
     int sa, sb;
@@ -1866,7 +1869,7 @@ int taps_fd_prepare_enqueue(taps_problem* P, int solver, int M, std::vector<FdPe
     }
     FdEntry* E = nullptr;
     FdPending T;
-    TAPS_TRY(fd_enqueue(P, P->dims[d], sa >= 0 ? P->ops[d][sa] : -1, P->ops[d][sb], &E, &T));
+    TAPS_TRY(fd_enqueue(P, P->dims[d], sa >= 0 ? P->ops[d][sa] : -1, P->ops[d][sb], beside, &E, &T));
     if (T.E) pend->push_back(T);
     if (!P->d_pq[d]) {   // the problem's source vectors in the pencil's eigenbasis
       const int n = P->dims[d]->nf;
@@ -1893,7 +1896,7 @@ int taps_fd_prepare_finish(std::vector<FdPending>* pend) {
 
 int taps_fd_prepare_all(taps_problem* P, int solver, int M) {
   std::vector<FdPending> pend;
-  int st = taps_fd_prepare_enqueue(P, solver, M, &pend);
+  int st = taps_fd_prepare_enqueue(P, solver, M, false, &pend);
   int s2 = taps_fd_prepare_finish(&pend);
   return st != TAPS_OK ? st : s2;
 }

@@ -45,3 +45,28 @@ def test_sweep_over_pencil_sizes(T, n, s):
     # reduced systems' floor in the other tests of this kind
     tol = max(1e-10, 10 * 2.2e-16 * 16 * n * n / np.pi ** 2)
     assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b)
+
+
+def test_batch_set_up_over_pencil_sizes(T):
+    """Decompositions side by side (a batch): cluster tridiagonalisations of more entries than a
+    CTA has threads, in distributed shared memory and in global memory."""
+    sizes = [300, 515, 560, 600, 644, 660, 700, 1000]
+    Ps, Us, descs, U0s = [], [], [], []
+    for n in sizes * 2:
+        dims = [W.dim(n), W.dim(9)]
+        rng = np.random.default_rng(n)
+        sources = [(1.0, [("nodal", rng.uniform(-1, 1, dm["n"])) for dm in dims]) for _ in range(4)]
+        desc = dict(name="pencil", dims=dims, terms=[(1.0, ["K", "M"]), (1.0, ["M", "K"])], sources=sources)
+        U0 = W.random_factors(desc, 3, seed=n)
+        stream = torch.cuda.Stream()
+        P = T.Problem(desc, stream=T.ctypes.c_void_p(stream.cuda_stream))
+        U = P.factors(3)
+        U.set(U0)
+        Ps.append(P), Us.append(U), descs.append((desc, stream)), U0s.append(U0)
+    T.Batch(Ps, Us, solver=T.SOLVER_FASTDIAG).sweep(1)
+    torch.cuda.synchronize()
+    for n, (desc, _), U, U0 in zip(sizes, descs, Us, U0s):
+        Uo, _ = O.sweep(O.problem_from_description(desc), [u.copy() for u in U0])
+        a, b = O.cp_full(U.get()), O.cp_full(Uo)
+        tol = max(1e-10, 10 * 2.2e-16 * 16 * n * n / np.pi ** 2)   # as above
+        assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b), n
