@@ -10,13 +10,13 @@
 // so a solve costs two n x n x M products and n small LU solves instead of a
 // sequential block elimination over the n block rows.
 //
-// The one-off pencil decomposition, in FP64: banded Cholesky B = L L^T and
-// S = L^{-1} A L^{-T} in one CTA, Householder tridiagonalisation S = Q T Q^T on one
-// thread-block cluster; then, in parallel, the eigenvalues of T by Sturm-count multisection (one warp per
-// eigenvalue), its eigenvectors by inverse iteration (one thread per eigenvector, one
-// per cluster of nearly equal eigenvalues), one step of symmetric orthogonalisation,
-// the back-transform Z = Q Z_T (one warp per column), and Phi = L^{-T} Z (one thread per
-// column).
+// The one-off pencil decomposition, in FP64: banded Cholesky B = L L^T on one warp,
+// S = L^{-1} A L^{-T} (one thread per column), Householder tridiagonalisation S = Q T Q^T on
+// one thread-block cluster or on all SMs; then, in parallel, the eigenvalues of T by
+// Sturm-count multisection (one warp per eigenvalue), its eigenvectors by inverse iteration
+// (one thread per eigenvector, one per cluster of nearly equal eigenvalues), one step of
+// symmetric orthogonalisation, the back-transform Z = Q Z_T (one warp per column), and
+// Phi = L^{-T} Z (one thread per column).
 #include <string.h>
 
 #include <algorithm>
@@ -1694,7 +1694,7 @@ static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, bool besi
     int tk = prof_begin(P, TAPS_PROF_OTHER);
     fd_dense_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(bandA, bandB, n, dm->hb, A, B);
     if (cudaMemsetAsync(V, 0, sizeof(double) * nn, s) != cudaSuccess) { st = TAPS_ERR_CUDA; break; }
-    // banded Cholesky and S, then the tridiagonalisation (one cluster)
+    // banded Cholesky and S, then the tridiagonalisation
     double* linv = T->tmp + n;   // the tridiagonalisation uses the first n
     if ((st = fd_cholesky(bandB, B, n, dm->hb, linv, P->d_status, maxsm_optin, s)) != TAPS_OK) break;
     if (hasA) {
