@@ -4,7 +4,7 @@
 // either side of the diagonal.  Its elimination is a chain of n dependent block rows, and
 // on this GPU the chain, not the FP64 work, is what a solve costs (64 nodes, 10 modes:
 // 3.8 MFLOP, 3 us at the FP64 peak; the one-ended cooperative elimination, two grid
-// barriers per row, took 1270 us with its back substitution).  Here:
+// barriers per row, takes 1150 us with its back substitution).  Here:
 //   - the chain is halved: one cluster eliminates the nodes from the low end, another the
 //     nodes from the high end, until hb nodes are left in the middle, to which both sides'
 //     Schur updates are added; a third cluster solves the middle and substitutes back
@@ -13,7 +13,7 @@
 //   - a row costs one hardware cluster barrier instead of two grid barriers through global
 //     memory.  The active window (hb + 1 nodes) lives in the cluster's shared memory, its
 //     scalar columns dealt out to the CTAs; per node k every CTA forms W = D^-1 A(k, .) for
-//     its own columns (reducing the diagonal block redundantly: M dependent pivots either
+//     its own columns (factoring the diagonal block redundantly: M dependent pivots either
 //     way) and subtracts A(., k) W from them.  The columns
 //     of node k + 1 are updated first and pushed to every CTA of the cluster (distributed
 //     shared memory), so the barrier's wait overlaps the rest of the update.
@@ -24,6 +24,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -94,23 +95,30 @@ struct TsArgs {
   int* status;
 };
 
-// W = D^-1 A(k, .) for the own columns of the window by Gauss-Jordan elimination without
-// pivoting on [D | own columns] (no inverse is formed: D^-1 A as a product would lose another
-// factor cond(D)).  Four warps, one per SM sub-partition: an FP64 instruction holds its
-// sub-partition's pipe ~64 clocks, and a second warp's would sit in the pivot chain (eight
-// warps took 1240 clocks a pivot at M = 10).  Warp w holds the columns w, w + 4, ... with the
-// rows on the lanes (S row slots).  Per step everyone reads the multipliers published by the
-// pivot's owner; the owner of the next column updates that column first and publishes its
-// multipliers (reciprocal by seed and refinement), the chain of the step.  After four pivots
+// W = D^-1 A(k, .) for the own columns of the window by LU without pivoting on [D | own
+// columns], row p divided by its pivot (no inverse is formed: D^-1 A as a product would lose
+// another factor cond(D); and the rows above a pivot wait for the back substitution: eliminated
+// at once, Gauss-Jordan, they leave residuals that grow with cond(D), 1e-13 where these are
+// 4e-17 on a 24-mode block of condition 7e12).  Four warps, one per SM sub-partition: an FP64
+// instruction holds its sub-partition's pipe ~64 clocks, and a second warp's would sit in the
+// pivot chain (eight warps took 1240 clocks a pivot at M = 10).  Warp w holds the columns w,
+// w + 4, ... with the rows on the lanes (S row slots).  Per step everyone reads the multipliers
+// published by the pivot's owner; the owner of the next column updates that column first and
+// publishes its multipliers (reciprocal by seed and refinement), the chain of the step, and its
+// entries above the diagonal, final by then, for the back substitution.  After four pivots
 // every warp's columns move down one register slot, so that the next pivot's column has a
-// fixed place.
-// get(ci, row): entry of own column ci (ncol of them); put(ci, row, w): its solution.
+// fixed place.  The back substitution needs no barrier: every warp takes its own columns through
+// the published ones of U, whose diagonal is one.  It is the price of the small residual: 64
+// nodes at s = 2 take 256 us a solve with it at M = 10 and 234 as Gauss-Jordan, 1280 and 1125 at
+// M = 30.
+// up[c * ld + r]: U above the diagonal, in the place of D, which is in registers by then.
+// put(ci, row, w): the solution of own column ci (ncol of them).
 __device__ __forceinline__ void ts_sync4(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
 __device__ __forceinline__ void ts_arrive4(int id) { asm volatile("bar.arrive %0, 128;" ::"r"(id) : "memory"); }
 
 template <int S, typename Put>
-__device__ __forceinline__ void ts_solve_node(double (&v)[TS_COLS / 4][S], int M, int ncol, double* colb, int* status,
-                                              bool report, Put put) {
+__device__ __forceinline__ void ts_solve_node(double (&v)[TS_COLS / 4][S], int M, int ncol, double* colb, double* up,
+                                              int ld, int* status, bool report, Put put) {
   constexpr int KC = TS_COLS / 4;
   const int lane = threadIdx.x & 31;
   const int w = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);   // the same in every lane: uniform branches
@@ -123,21 +131,24 @@ __device__ __forceinline__ void ts_solve_node(double (&v)[TS_COLS / 4][S], int M
     }
     return rp;
   };
-  // every row less its multiplier times row p; row p times the reciprocal
+  // every row below p less its multiplier times row p; row p times the reciprocal
   auto update = [&](double (&x)[S], const double (&f)[S], int p) {
     const double rp = row_of(x, p);
 #pragma unroll
     for (int s = 0; s < S; ++s) x[s] = fma(-f[s], rp, lane + 32 * s == p ? 0.0 : x[s]);
   };
-  auto publish = [&](const double (&x)[S], int q) {   // the multipliers of pivot q; -1 / pivot in its row
+  // the multipliers of pivot q, none above it; -1 / pivot in its row; U above it
+  auto publish = [&](const double (&x)[S], int q) {
     const double piv = row_of(x, q);
     double inv = taps_rcp(piv);
     const bool ok = taps_finite_nonzero(piv);
     if (!ok) inv = 1.0;
 #pragma unroll
     for (int s = 0; s < S; ++s) {
+      const int r = lane + 32 * s;
       const double f = x[s] * inv;
-      colb[(q & 1) * 64 + lane + 32 * s] = lane + 32 * s == q ? -inv : f;
+      colb[(q & 1) * 64 + r] = r < q ? 0.0 : (r == q ? -inv : f);
+      if (r < q) up[q * ld + r] = x[s];
     }
     if (!ok && report && lane == 0) taps_flag(status, TAPS_DEV_SINGULAR);
   };
@@ -199,13 +210,78 @@ __device__ __forceinline__ void ts_solve_node(double (&v)[TS_COLS / 4][S], int M
       c0 += 4;
     }
   }
+  // back substitution: the rows above r less U(., r) times row r, for the slots that hold own
+  // columns (the first may hold one of D's), U's next column loaded ahead
+  if (c0 < M) {
+#pragma unroll
+    for (int k = 0; k + 1 < KC; ++k)
+#pragma unroll
+      for (int s = 0; s < S; ++s) v[k][s] = v[k + 1][s];
+    c0 += 4;
+  }
+  const int held = (tot - c0 + 3) >> 2;
+  if (S == 1 && M <= 16) {
+    // two columns to a slot, one to a half of the lanes: an FP64 instruction costs the same
+    const int row = lane & 15, top = lane & 16;
+    double x[KC / 2];
+#pragma unroll
+    for (int k = 0; k < KC / 2; ++k) {
+      const double hi = __shfl_sync(0xffffffffu, v[2 * k + 1][0], row);
+      x[k] = top ? hi : v[2 * k][0];
+    }
+    auto back = [&](auto slots) {
+      double u = row < M - 1 ? up[(M - 1) * ld + row] : 0.0;
+#pragma unroll 1
+      for (int r = M - 1; r > 0; --r) {
+        const double ur = u;
+        u = row < r - 1 ? up[(r - 1) * ld + row] : 0.0;
+#pragma unroll
+        for (int k = 0; k < decltype(slots)::value; ++k)
+          x[k] = fma(-ur, __shfl_sync(0xffffffffu, x[k], r + top), x[k]);
+      }
+    };
+    if (held > 4) back(std::integral_constant<int, KC / 2>{});
+    else if (held > 2) back(std::integral_constant<int, 2>{});
+    else if (held > 0) back(std::integral_constant<int, 1>{});
+#pragma unroll
+    for (int k = 0; k < KC / 2; ++k) {
+      const int c = c0 + 8 * k + (top >> 2);
+      if (row < M && c < tot) put(c - M, row, x[k]);
+    }
+    return;
+  }
+  auto back = [&](auto slots) {
+    double u[S];
+#pragma unroll
+    for (int s = 0; s < S; ++s) u[s] = lane + 32 * s < M - 1 ? up[(M - 1) * ld + lane + 32 * s] : 0.0;
+#pragma unroll 1
+    for (int r = M - 1; r > 0; --r) {
+      double ur[S];
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        ur[s] = u[s];
+        u[s] = lane + 32 * s < r - 1 ? up[(r - 1) * ld + lane + 32 * s] : 0.0;
+      }
+#pragma unroll
+      for (int k = 0; k < decltype(slots)::value; ++k) {
+        const double xr = row_of(v[k], r);
+#pragma unroll
+        for (int s = 0; s < S; ++s)
+          if (s == 0 || r > 32) v[k][s] = fma(-ur[s], xr, v[k][s]);
+      }
+    }
+  };
+  if (held > 4) back(std::integral_constant<int, KC>{});
+  else if (held > 3) back(std::integral_constant<int, 4>{});
+  else if (held > 2) back(std::integral_constant<int, 3>{});
+  else if (held > 0) back(std::integral_constant<int, 2>{});
 #pragma unroll
   for (int k = 0; k < KC; ++k) {
     const int c = c0 + 4 * k;
 #pragma unroll
     for (int s = 0; s < S; ++s) {
       const int r = lane + 32 * s;
-      if (r < M && c >= M && c < tot) put(c - M, r, v[k][s]);
+      if (r < M && c < tot) put(c - M, r, v[k][s]);
     }
   }
 }
@@ -323,7 +399,7 @@ __device__ __forceinline__ void ts_eliminate(const TsArgs& a, int base, int dir,
           if (lane + 32 * s < M) v[q][s] = x[lane + 32 * s];
       }
       __syncthreads();
-      ts_solve_node<S>(v, M, nall, sm + L.col, a.status, rank == 0, [&](int ci, int m, double w) {
+      ts_solve_node<S>(v, M, nall, sm + L.col, pan, rows, a.status, rank == 0, [&](int ci, int m, double w) {
         const int g = g0 + (ci << sh);
         wbuf[ci * M + m] = w;
         if (ci < ncol) *const_cast<double*>(node_addr(k, byM.div(g), m, byM.mod(g))) = w;
@@ -532,8 +608,8 @@ static bool ts_fits(int hb, int M, int nc, size_t smem) {
 
 // CTAs per cluster: the largest the device places, unless a CTA would hold fewer than four
 // of the window's columns.  Measured per solve (elimination, middle, back substitution, us,
-// 64 nodes, hb = 5) with 4 / 8 / 16 CTAs: M = 6: 195 / 181 / 176, M = 10: 335 / 271 / 238,
-// M = 20: 1035 / 739 / 574, M = 30: - / 1552 / 1116; 16 nodes, M = 4: 51 / 50 / 51.
+// 64 nodes, hb = 5) with 4 / 8 / 16 CTAs: M = 6: 205 / 188 / 180, M = 10: 367 / 288 / 256,
+// M = 20: 1583 / 869 / 656, M = 30: - / 2355 / 1280; 14 nodes, M = 4: 52 / 51 / 51.
 static int ts_cluster_size(int hb, int M, int most) {
   int nc = 1;
   while (nc < most && (hb + 1) * M > 4 * nc) nc *= 2;
@@ -612,9 +688,12 @@ int taps_ts_setup(int maxsm, int* most, size_t* smem) {
 }
 
 // CTAs per cluster for a dim of half-bandwidth hb at M modes; 0: the one-ended route.
-// Beyond hb = 5 (s >= 3) the one-ended elimination stays: both are equally accurate, but
-// fixed-M iterations on the third-order spaces end where rounding takes them (the space-time
-// refinement study at s = p = 3, 30 modes, 400 nodes: error 4.2e-7 one way, 9.1e-7 the other).
+// Beyond hb = 5 (s >= 3) the one-ended elimination stays, to keep the results that users of
+// those spaces have: not for accuracy (backward errors of single solves, 32 nodes, 6 and 12 modes
+// with two of them 1e-5 apart, from both ends / from one: s = 2: 5.6e-14, 1.0e-13 / 8.4e-14,
+// 1.1e-13; s = 3: 7.2e-14, 1.1e-13 / 8.6e-14, 1.3e-13) nor for speed (64 nodes of 10 modes at
+// s = 3: 294 us / 1240 us), but because fixed-M iterations at third order end where rounding takes
+// them, and the order that the space-time refinement study shows at s = p = 3 depends on it.
 int taps_ts_ctas(const taps_problem* P, int hb, int M) {
   if (hb > 5 || M > 64 || P->ts_most < 1) return 0;
   int nc = ts_cluster_size(hb, M, P->ts_most);
