@@ -1561,7 +1561,7 @@ extern "C" int taps_batch_create(taps_problem* const* probs, taps_factors* const
       for (int i = i0; i < i1 && st == TAPS_OK; ++i) {
         if ((st = taps_ws_ensure(B->P[i], B->U[i]->M)) != TAPS_OK) break;
         // FASTDIAG's pencils cover MODEDIAG's (the dims it cannot solve on the mode side)
-        st = taps_fd_prepare_enqueue(B->P[i], B->eff_solver, B->U[i]->M, B->count > 1, &pend);
+        st = taps_fd_prepare_enqueue(B->P[i], B->eff_solver, B->U[i]->M, &pend);
       }
       int s2 = taps_fd_prepare_finish(&pend);
       if (st == TAPS_OK) st = s2;

@@ -1538,28 +1538,29 @@ static bool td_grid_ok(size_t smem, int maxsm) {
   return per_sm > 0;
 }
 
-// The tridiagonalisation of S (n x n in A): S in a cluster's distributed shared memory up to
-// TD_CLUSTER_MOST nodes, where its cheaper barriers win, then in the shared memory of all num_sms
-// SMs while its rows fit (152: n <= ~1820), else in global memory.  Cluster and chip: 1.75 and
-// 2.34 ms for 254 nodes, 3.55 and 3.69 for 382, 6.28 and 5.21 for 510, 10.4 and 6.78 for 638.
-// beside: a batch enqueues many instances' decompositions at once, and nine clusters side by side
-// do more of them than one chip-wide kernel after another (24 instances of three dims of 460 to
-// 640 nodes: 303 and 540 ms; of 700 to 1024: 1.05 and 1.20 s).
+// The tridiagonalisation of S (n x n in A): S in a cluster's distributed shared memory while its
+// rows fit (16 CTAs: n <= 656), then in the shared memory of all num_sms SMs while they fit (152:
+// n <= ~1820), else in global memory.  The dim's size alone decides: the decomposition is kept for
+// every later solve of the dim, which must not round differently for having come first from a
+// batch, and decompositions run side by side from a batch or from a caller's threads as well as
+// alone.  Decomposition and first solve of 18 instances in a batch / from 18 threads / of one
+// instance, ms, on clusters and on the whole chip: 449 nodes: 49, 93, 9.5 and 114, 122, 9.2; 640:
+// 109, 152, 18.8 and 175, 234, 15.0; 800 (a cluster's S in global memory): 225, 376, 41.8 and 251,
+// 326, 19.9; 1300: 778, 1073, 123 and 799, 844, 52; 1800: 1916, 2531, 272 and 1774, 1787, 104.
 // xch: 4 n doubles and two words of workspace.
-#define TD_CLUSTER_MOST 448
 static int td_run(double* A, double* V, double* tmp, double* bt, double* dd, double* ee, int n, int maxsm,
-                  int num_sms, bool beside, double* xch, int* status, cudaStream_t s) {
+                  int num_sms, double* xch, int* status, cudaStream_t s) {
   const size_t dsm16 = sizeof(double) * ((size_t)((n + 15) / 16) * n + 3 * (size_t)n);
   const size_t dsm8 = sizeof(double) * ((size_t)((n + 7) / 8) * n + 3 * (size_t)n);
   const size_t gsm = sizeof(double) * 3 * (size_t)n;
   const size_t grd = sizeof(double) * ((size_t)((n + num_sms - 1) / num_sms) * n + 3 * (size_t)n);
   cudaError_t ce;
-  const bool small = beside || n <= TD_CLUSTER_MOST || grd + 1024 > (size_t)maxsm || n > TDG_THREADS * TDG_PER;
-  if (small && dsm16 + 1024 <= (size_t)maxsm && td_cluster_ok<16>((const void*)fd_tridiag_dsmem_kernel<16>, dsm16, TDS_THREADS)) {
+  const bool chip = grd + 1024 <= (size_t)maxsm && n <= TDG_THREADS * TDG_PER;
+  if (dsm16 + 1024 <= (size_t)maxsm && td_cluster_ok<16>((const void*)fd_tridiag_dsmem_kernel<16>, dsm16, TDS_THREADS)) {
     ce = td_launch<16>(fd_tridiag_dsmem_kernel<16>, TDS_THREADS, dsm16, s, (const double*)A, V, bt, dd, ee, n);
-  } else if (small && dsm8 + 1024 <= (size_t)maxsm && td_cluster_ok<8>((const void*)fd_tridiag_dsmem_kernel<8>, dsm8, TDS_THREADS)) {
+  } else if (dsm8 + 1024 <= (size_t)maxsm && td_cluster_ok<8>((const void*)fd_tridiag_dsmem_kernel<8>, dsm8, TDS_THREADS)) {
     ce = td_launch<8>(fd_tridiag_dsmem_kernel<8>, TDS_THREADS, dsm8, s, (const double*)A, V, bt, dd, ee, n);
-  } else if (!small && td_grid_ok(grd, maxsm)) {
+  } else if (chip && td_grid_ok(grd, maxsm)) {
     unsigned* bar = reinterpret_cast<unsigned*>(xch + 4 * (size_t)n);
     TAPS_CUDA(cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), s));
     const double* Ac = A;
@@ -1638,7 +1639,7 @@ static int iv_launch(const double* dd, const double* ee, const double* lam, int 
 // waiting for it: the entry is registered at once (pending, with an event recorded
 // after its last kernel) and the temporaries are returned in *T for fd_finish.  An
 // entry that already exists, pending on another stream, makes P's stream wait for it.
-static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, bool beside, FdEntry** out, FdPending* T) {
+static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, FdEntry** out, FdPending* T) {
   memset(T, 0, sizeof(*T));
   for (int k = 0; k < dm->nfd; ++k)
     if (dm->fd[k].opA == opA && dm->fd[k].opB == opB) {
@@ -1703,7 +1704,7 @@ static int fd_enqueue(taps_problem* P, taps_dim* dm, int opA, int opB, bool besi
       if ((st = fd_lsolve(B, linv, V, n, dm->hb, 1, W, s)) != TAPS_OK) break;
       fd_symmetrize_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(W, n, A);
       if (cudaMemsetAsync(V, 0, sizeof(double) * nn, s) != cudaSuccess) { st = TAPS_ERR_CUDA; break; }
-      if ((st = td_run(A, V, T->tmp, T->bt, T->dd, T->ee, n, maxsm_optin, P->num_sms, beside, W, P->d_status, s)) != TAPS_OK) break;
+      if ((st = td_run(A, V, T->tmp, T->bt, T->dd, T->ee, n, maxsm_optin, P->num_sms, W, P->d_status, s)) != TAPS_OK) break;
       // eigenvalues (warp each), eigenvectors (thread each), back-transform (warp each),
       // all into A, which the tridiagonalisation no longer needs
       // two warps per CTA: the warps' FP64 chains spread over the SMs' sub-partitions
@@ -1775,7 +1776,7 @@ static int fd_finish(FdPending& T) {
 static int fd_prepare(taps_problem* P, int d, taps_dim* dm, int opA, int opB, FdEntry** out) {
   (void)d;
   FdPending T;
-  int st = fd_enqueue(P, dm, opA, opB, false, out, &T);
+  int st = fd_enqueue(P, dm, opA, opB, out, &T);
   if (st != TAPS_OK) return st;
   return fd_finish(T);
 }
@@ -1856,7 +1857,7 @@ int taps_fd_to_nodal(taps_problem* P, const FdEntry* E, const double* Y, int n, 
 // their temporaries in *pend; the finish half waits, checks and frees.  Batches
 // enqueue many problems (each on its own stream) before finishing any, so the
 // decompositions of different instances run concurrently.
-int taps_fd_prepare_enqueue(taps_problem* P, int solver, int M, bool beside, std::vector<FdPending>* pend) {
+int taps_fd_prepare_enqueue(taps_problem* P, int solver, int M, std::vector<FdPending>* pend) {
   if (solver != TAPS_SOLVER_FASTDIAG && solver != TAPS_SOLVER_MODEDIAG) return TAPS_OK;
   for (int d = 0; d < P->D; ++d) {
     int sa, sb;
@@ -1869,7 +1870,7 @@ int taps_fd_prepare_enqueue(taps_problem* P, int solver, int M, bool beside, std
     }
     FdEntry* E = nullptr;
     FdPending T;
-    TAPS_TRY(fd_enqueue(P, P->dims[d], sa >= 0 ? P->ops[d][sa] : -1, P->ops[d][sb], beside, &E, &T));
+    TAPS_TRY(fd_enqueue(P, P->dims[d], sa >= 0 ? P->ops[d][sa] : -1, P->ops[d][sb], &E, &T));
     if (T.E) pend->push_back(T);
     if (!P->d_pq[d]) {   // the problem's source vectors in the pencil's eigenbasis
       const int n = P->dims[d]->nf;
@@ -1896,7 +1897,7 @@ int taps_fd_prepare_finish(std::vector<FdPending>* pend) {
 
 int taps_fd_prepare_all(taps_problem* P, int solver, int M) {
   std::vector<FdPending> pend;
-  int st = taps_fd_prepare_enqueue(P, solver, M, false, &pend);
+  int st = taps_fd_prepare_enqueue(P, solver, M, &pend);
   int s2 = taps_fd_prepare_finish(&pend);
   return st != TAPS_OK ? st : s2;
 }

@@ -456,8 +456,7 @@ size_t taps_fdw_scratch_doubles(int nf_max, int M);
 int taps_fdw_solve(taps_problem* P, taps_factors* U, int d);
 int taps_fd_lookup(taps_problem* P, int d, int opA, int opB, const FdEntry** out);
 int taps_fd_to_nodal(taps_problem* P, const FdEntry* E, const double* Y, int n, int M, double* Out, double* Save);
-// beside: other decompositions are enqueued on other streams (a batch).
-int taps_fd_prepare_enqueue(taps_problem* P, int solver, int M, bool beside, std::vector<FdPending>* pend);
+int taps_fd_prepare_enqueue(taps_problem* P, int solver, int M, std::vector<FdPending>* pend);
 int taps_fd_prepare_finish(std::vector<FdPending>* pend);
 int taps_lu_needs_tuning(const taps_problem* P, int solver, int M);
 int taps_check_status(int* d_status, cudaStream_t s);
