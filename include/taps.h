@@ -369,7 +369,10 @@ int taps_eval_grid_noalloc(const taps_problem* prob, const taps_factors* U, cons
                            const int* count, const int* step, void* out_dev, int out_dtype);
 /* Points: u^TD(x) = sum_m prod_d sum_I N~_I(x_d) U_d[I, m] at n_pts points; pts_dev is
  * device memory [n_pts][D] row-major (coordinates clamped to [lo, hi]); out_dev
- * receives n_pts FP64 values.  Asynchronous on the problem's stream. */
+ * receives n_pts FP64 values.  Asynchronous on the problem's stream.  The first call on a
+ * factor set may allocate device memory for its per-element polynomials (10 doubles per
+ * element, dim and pair of modes of its capacity), which stays until the factors are destroyed;
+ * where there is none, or that call is being captured, the points are evaluated without. */
 int taps_eval_points(const taps_problem* prob, const taps_factors* U, int n_pts,
                      const double* pts_dev, double* out_dev);
 

@@ -870,8 +870,17 @@ static double* ep_tables(const taps_problem* P, taps_factors* U) {
   }
   size_t tot = 0;
   for (int d = 0; d < P->D; ++d) tot += (size_t)(P->dims[d]->n - 1) * ((U->M_cap + 1) / 2) * (2 * EP_Q);
+  // an allocation is a prohibited call, and ends the capture, while any stream is being captured
+  // in the global mode; this one touches no captured stream, so it is made in the relaxed mode
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
   double* p = nullptr;
-  if (taps_alloc((void**)&p, sizeof(double) * tot) != TAPS_OK) {
+  const int st = taps_alloc((void**)&p, sizeof(double) * tot);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (st != TAPS_OK) {
     cudaGetLastError();
     return nullptr;
   }
