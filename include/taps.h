@@ -468,7 +468,8 @@ int taps_factors_from_profiles(const taps_problem* prob, taps_factors* U, int M,
 #define TAPS_PROF_GRAM 0          /* fused banded SpMM + Gram (partial + reduce)   */
 #define TAPS_PROF_COEFF 1         /* Hadamard coefficient combine                   */
 #define TAPS_PROF_BLOCK_ASSEMBLE 2 /* reduced block band + right-hand side          */
-#define TAPS_PROF_BLOCK_LU 3      /* cooperative block-banded elimination           */
+#define TAPS_PROF_BLOCK_LU 3      /* block-banded elimination: the cooperative one, or the
+                                     middle and back substitution of the two-sided one */
 #define TAPS_PROF_BACKSUB 4       /* block back substitution                        */
 #define TAPS_PROF_NORMALIZE 5     /* column normalisation + factor change           */
 #define TAPS_PROF_RESIDUAL 6      /* residual kernels                               */
@@ -478,7 +479,8 @@ int taps_factors_from_profiles(const taps_problem* prob, taps_factors* U, int M,
 #define TAPS_PROF_FD_TRANSFORM 10 /* fast diagonalisation: back to the nodal basis   */
 #define TAPS_PROF_MODEDIAG 11     /* mode-side diagonalisation: M x M eigenproblem,
                                      banded solves, transform                       */
-#define TAPS_PROF_NUM 12
+#define TAPS_PROF_BLOCK_ENDS 12   /* two-sided elimination: from both ends to the middle */
+#define TAPS_PROF_NUM 13
 int taps_profile_reset(taps_problem* prob, int enable_events);
 int taps_profile_get(taps_problem* prob, int kernel_class, long long* launches, double* ms,
                      double* flops, double* bytes);

@@ -1156,10 +1156,7 @@ static int reduced_solve_block_lu(taps_problem* P, taps_factors* U, int d) {
   const double band_bytes = 8.0 * (double)nf * nb * M * M;
   const int nc = taps_ts_ctas(P, hb, M);
   if (nc > 0) {   // from both ends, middle and back substitution; keeps the old factor in d_Uold
-    tk = prof_begin(P, TAPS_PROF_BLOCK_LU);
-    TAPS_TRY(taps_ts_solve(P, U, d, nc));
-    prof_end(P, TAPS_PROF_BLOCK_LU, tk, lu_flops + bs_flops, 2.0 * band_bytes + 16.0 * nf * M);
-    return TAPS_OK;
+    return taps_ts_solve(P, U, d, nc, lu_flops, bs_flops, 2.0 * band_bytes + 16.0 * nf * M);
   }
   TAPS_CUDA(cudaMemcpyAsync(P->d_Uold, U->d_U[d], sizeof(double) * nf * M, cudaMemcpyDeviceToDevice, s));
   // cooperative elimination; the CTA count comes from the tuner (first use per (n, M))

@@ -465,7 +465,7 @@ int taps_check_status(int* d_status, cudaStream_t s);
 int taps_ts_setup(int maxsm, int* most, size_t* smem);
 int taps_ts_ctas(const taps_problem* P, int hb, int M);
 size_t taps_ts_scratch_doubles(int hb, int M);
-int taps_ts_solve(taps_problem* P, taps_factors* U, int d, int nc);
+int taps_ts_solve(taps_problem* P, taps_factors* U, int d, int nc, double lu_flops, double bs_flops, double bytes);
 int taps_fd_eligible(const taps_problem* P, int d, int* slotA, int* slotB);
 // F[i][m] = sum_r q[r][i] c[r][m] (q [Rf][n], c [Rf][M], F [n][M]).
 int taps_rhs(const double* q, const double* c, int Rf, int n, int M, double* F, int num_sms, cudaStream_t s);

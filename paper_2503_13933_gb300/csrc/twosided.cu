@@ -704,8 +704,9 @@ int taps_ts_ctas(const taps_problem* P, int hb, int M) {
 size_t taps_ts_scratch_doubles(int hb, int M) { return 2 * ((size_t)hb * M + 1) * hb * M; }
 
 // Solves the reduced system of dim d assembled in P->d_blocks / P->d_F; the factor before
-// the solve goes to P->d_Uold.
-int taps_ts_solve(taps_problem* P, taps_factors* U, int d, int nc) {
+// the solve goes to P->d_Uold.  The profile counts the ends' kernel (with the elimination's flops
+// and the bytes) and the middle's apart.
+int taps_ts_solve(taps_problem* P, taps_factors* U, int d, int nc, double lu_flops, double bs_flops, double bytes) {
   const taps_dim* dm = P->dims[d];
   TsArgs a;
   memset(&a, 0, sizeof(a));
@@ -723,13 +724,16 @@ int taps_ts_solve(taps_problem* P, taps_factors* U, int d, int nc) {
   a.status = P->d_status;
   const bool wide = a.M > 32;
   size_t smem = ts_smem_bytes(a.hb, a.M, nc);
-  if (a.nlo > 0) {
+  const bool ends = a.nlo > 0;
+  if (ends) {
+    const int tk = prof_begin(P, TAPS_PROF_BLOCK_ENDS);
     const cudaError_t ce = ts_launch(wide ? ts_sides_kernel<2> : ts_sides_kernel<1>, (a.nhi > 0 ? 2 : 1) * nc, nc, smem,
                                      P->stream, a);
     if (ce != cudaSuccess) {
       taps_note_cuda_error(ce, "two-sided elimination launch", __FILE__, __LINE__);
       return TAPS_ERR_CUDA;
     }
+    prof_end(P, TAPS_PROF_BLOCK_ENDS, tk, lu_flops, bytes);
   }
   // the back substitution's stages share the elimination's shared memory
   const size_t rows = 2 * (size_t)(a.hb + 1) * a.M, stage = (size_t)a.hb * a.M * a.M + a.M;
@@ -738,11 +742,13 @@ int taps_ts_solve(taps_problem* P, taps_factors* U, int d, int nc) {
   smem = std::max(smem, sizeof(double) * (rows + stages * stage));
   const int fnc = std::max(nc, std::min(2, P->ts_most));
   smem = std::max(smem, ts_smem_bytes(a.hb, a.M, fnc));
+  const int tk = prof_begin(P, TAPS_PROF_BLOCK_LU);
   const cudaError_t ce =
       ts_launch_finish(wide ? ts_finish_kernel<2> : ts_finish_kernel<1>, fnc, smem, P->stream, a, stages);
   if (ce != cudaSuccess) {
     taps_note_cuda_error(ce, "middle and back substitution launch", __FILE__, __LINE__);
     return TAPS_ERR_CUDA;
   }
+  prof_end(P, TAPS_PROF_BLOCK_LU, tk, ends ? bs_flops : lu_flops + bs_flops, ends ? 0.0 : bytes);
   return TAPS_OK;
 }

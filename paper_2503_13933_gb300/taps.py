@@ -142,7 +142,7 @@ SIGNATURES = {
 }
 
 PROF_CLASSES = ["gram", "coeff", "block_assemble", "block_lu", "backsub", "normalize",
-                "residual", "eval", "other", "fastdiag", "fd_transform", "modediag"]
+                "residual", "eval", "other", "fastdiag", "fd_transform", "modediag", "block_ends"]
 
 _LIB = None
 
