@@ -96,21 +96,21 @@ struct TsArgs {
 };
 
 // W = D^-1 A(k, .) for the own columns of the window by LU without pivoting on [D | own
-// columns], row p divided by its pivot (no inverse is formed: D^-1 A as a product would lose
-// another factor cond(D); and the rows above a pivot wait for the back substitution: eliminated
-// at once, Gauss-Jordan, they leave residuals that grow with cond(D), 1e-13 where these are
-// 4e-17 on a 24-mode block of condition 7e12).  Four warps, one per SM sub-partition: an FP64
-// instruction holds its sub-partition's pipe ~64 clocks, and a second warp's would sit in the
-// pivot chain (eight warps took 1240 clocks a pivot at M = 10).  Warp w holds the columns w,
-// w + 4, ... with the rows on the lanes (S row slots).  Per step everyone reads the multipliers
-// published by the pivot's owner; the owner of the next column updates that column first and
-// publishes its multipliers (reciprocal by seed and refinement), the chain of the step, and its
-// entries above the diagonal, final by then, for the back substitution.  After four pivots
-// every warp's columns move down one register slot, so that the next pivot's column has a
-// fixed place.  The back substitution needs no barrier: every warp takes its own columns through
-// the published ones of U, whose diagonal is one.  It is the price of the small residual: 64
-// nodes at s = 2 take 256 us a solve with it at M = 10 and 234 as Gauss-Jordan, 1280 and 1125 at
-// M = 30.
+// columns] (no inverse is formed: D^-1 A as a product would lose another factor cond(D); and the
+// rows above a pivot wait for the back substitution: eliminated at once, Gauss-Jordan, they
+// leave residuals that grow with cond(D), 8e-14 where these are 2e-17 on a 24-mode block of
+// condition 2e15).  Every entry takes the operations of the one-ended elimination in their
+// order.  Four warps, one per SM sub-partition: an FP64 instruction holds its
+// sub-partition's pipe ~64 clocks, and a second warp's would sit in the pivot chain (eight warps
+// took 1240 clocks a pivot at M = 10).  Warp w holds the columns w, w + 4, ... with the rows on
+// the lanes (S row slots).  Per step everyone reads the multipliers published by the pivot's
+// owner; the owner of the next column updates that column first and publishes its multipliers
+// (reciprocal by seed and refinement), the chain of the step, and its entries above the
+// diagonal, final by then, for the back substitution.  After four pivots every warp's columns
+// move down one register slot, so that the next pivot's column has a fixed place.  The back
+// substitution needs no barrier: every warp takes its own columns through the published ones of
+// U, with the kept reciprocals of its diagonal.  It is the price of the small residual: 64 nodes
+// at s = 2 take 266 us a solve at M = 10 and 234 as Gauss-Jordan, 1372 and 1125 at M = 30.
 // up[c * ld + r]: U above the diagonal, in the place of D, which is in registers by then.
 // put(ci, row, w): the solution of own column ci (ncol of them).
 __device__ __forceinline__ void ts_sync4(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
@@ -123,6 +123,7 @@ __device__ __forceinline__ void ts_solve_node(double (&v)[TS_COLS / 4][S], int M
   const int lane = threadIdx.x & 31;
   const int w = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);   // the same in every lane: uniform branches
   const int tot = M + ncol;
+  double rinv[S] = {};   // 1 / pivot of the lane's rows
   auto row_of = [&](const double (&x)[S], int p) {
     double rp = __shfl_sync(0xffffffffu, x[0], p & 31);
     if (S > 1) {
@@ -131,13 +132,13 @@ __device__ __forceinline__ void ts_solve_node(double (&v)[TS_COLS / 4][S], int M
     }
     return rp;
   };
-  // every row below p less its multiplier times row p; row p times the reciprocal
+  // every row below p less its multiplier times row p
   auto update = [&](double (&x)[S], const double (&f)[S], int p) {
     const double rp = row_of(x, p);
 #pragma unroll
-    for (int s = 0; s < S; ++s) x[s] = fma(-f[s], rp, lane + 32 * s == p ? 0.0 : x[s]);
+    for (int s = 0; s < S; ++s) x[s] = fma(-f[s], rp, x[s]);
   };
-  // the multipliers of pivot q, none above it; -1 / pivot in its row; U above it
+  // the multipliers of pivot q, none above it; 1 / pivot in its row; U above it
   auto publish = [&](const double (&x)[S], int q) {
     const double piv = row_of(x, q);
     double inv = taps_rcp(piv);
@@ -147,7 +148,7 @@ __device__ __forceinline__ void ts_solve_node(double (&v)[TS_COLS / 4][S], int M
     for (int s = 0; s < S; ++s) {
       const int r = lane + 32 * s;
       const double f = x[s] * inv;
-      colb[(q & 1) * 64 + r] = r < q ? 0.0 : (r == q ? -inv : f);
+      colb[(q & 1) * 64 + r] = r < q ? 0.0 : (r == q ? inv : f);
       if (r < q) up[q * ld + r] = x[s];
     }
     if (!ok && report && lane == 0) taps_flag(status, TAPS_DEV_SINGULAR);
@@ -178,7 +179,13 @@ __device__ __forceinline__ void ts_solve_node(double (&v)[TS_COLS / 4][S], int M
   auto step = [&](int p, int c0, double (&next)[S]) {
     double f[S];
 #pragma unroll
-    for (int s = 0; s < S; ++s) f[s] = colb[(p & 1) * 64 + lane + 32 * s];
+    for (int s = 0; s < S; ++s) {
+      f[s] = colb[(p & 1) * 64 + lane + 32 * s];
+      if (lane + 32 * s == p) {
+        rinv[s] = f[s];
+        f[s] = 0.0;
+      }
+    }
     const int q = p + 1;
     if (q < M && w == (q & 3)) {
       update(next, f, p);
@@ -229,15 +236,19 @@ __device__ __forceinline__ void ts_solve_node(double (&v)[TS_COLS / 4][S], int M
       const double hi = __shfl_sync(0xffffffffu, v[2 * k + 1][0], row);
       x[k] = top ? hi : v[2 * k][0];
     }
+    const double ri = __shfl_sync(0xffffffffu, rinv[0], row);
     auto back = [&](auto slots) {
       double u = row < M - 1 ? up[(M - 1) * ld + row] : 0.0;
 #pragma unroll 1
-      for (int r = M - 1; r > 0; --r) {
+      for (int r = M - 1; r >= 0; --r) {
         const double ur = u;
         u = row < r - 1 ? up[(r - 1) * ld + row] : 0.0;
 #pragma unroll
-        for (int k = 0; k < decltype(slots)::value; ++k)
-          x[k] = fma(-ur, __shfl_sync(0xffffffffu, x[k], r + top), x[k]);
+        for (int k = 0; k < decltype(slots)::value; ++k) {
+          const double xs = x[k] * ri, xr = __shfl_sync(0xffffffffu, xs, r + top);   // every lane
+          const double y = fma(-ur, xr, x[k]);
+          x[k] = row == r ? xs : y;
+        }
       }
     };
     if (held > 4) back(std::integral_constant<int, KC / 2>{});
@@ -255,19 +266,30 @@ __device__ __forceinline__ void ts_solve_node(double (&v)[TS_COLS / 4][S], int M
 #pragma unroll
     for (int s = 0; s < S; ++s) u[s] = lane + 32 * s < M - 1 ? up[(M - 1) * ld + lane + 32 * s] : 0.0;
 #pragma unroll 1
-    for (int r = M - 1; r > 0; --r) {
+    for (int r = M - 1; r >= 0; --r) {
       double ur[S];
 #pragma unroll
       for (int s = 0; s < S; ++s) {
         ur[s] = u[s];
         u[s] = lane + 32 * s < r - 1 ? up[(r - 1) * ld + lane + 32 * s] : 0.0;
       }
+      // row r of slot k in lane k: one product with the reciprocal for all slots
+      const double ir = row_of(rinv, r);
+      double xp = 0.0;
 #pragma unroll
       for (int k = 0; k < decltype(slots)::value; ++k) {
-        const double xr = row_of(v[k], r);
+        const double t = row_of(v[k], r);
+        if (lane == k) xp = t;
+      }
+      xp *= ir;
 #pragma unroll
-        for (int s = 0; s < S; ++s)
-          if (s == 0 || r > 32) v[k][s] = fma(-ur[s], xr, v[k][s]);
+      for (int k = 0; k < decltype(slots)::value; ++k) {
+        const double xr = __shfl_sync(0xffffffffu, xp, k);
+#pragma unroll
+        for (int s = 0; s < S; ++s) {
+          const double y = s == 0 || r > 32 ? fma(-ur[s], xr, v[k][s]) : v[k][s];
+          v[k][s] = lane + 32 * s == r ? xr : y;
+        }
       }
     }
   };
@@ -608,8 +630,8 @@ static bool ts_fits(int hb, int M, int nc, size_t smem) {
 
 // CTAs per cluster: the largest the device places, unless a CTA would hold fewer than four
 // of the window's columns.  Measured per solve (elimination, middle, back substitution, us,
-// 64 nodes, hb = 5) with 4 / 8 / 16 CTAs: M = 6: 205 / 188 / 180, M = 10: 367 / 288 / 256,
-// M = 20: 1583 / 869 / 656, M = 30: - / 2355 / 1280; 14 nodes, M = 4: 52 / 51 / 51.
+// 64 nodes, hb = 5) with 4 / 8 / 16 CTAs: M = 6: 219 / 194 / 187, M = 10: 398 / 303 / 266,
+// M = 20: 1731 / 958 / 696, M = 30: - / 2573 / 1372; 14 nodes, M = 4: 56 / 54 / 54.
 static int ts_cluster_size(int hb, int M, int most) {
   int nc = 1;
   while (nc < most && (hb + 1) * M > 4 * nc) nc *= 2;
@@ -690,9 +712,9 @@ int taps_ts_setup(int maxsm, int* most, size_t* smem) {
 // CTAs per cluster for a dim of half-bandwidth hb at M modes; 0: the one-ended route.
 // Beyond hb = 5 (s >= 3) the one-ended elimination stays, to keep the results that users of
 // those spaces have: not for accuracy (backward errors of single solves, 32 nodes, 6 and 12 modes
-// with two of them 1e-5 apart, from both ends / from one: s = 2: 5.6e-14, 1.0e-13 / 8.4e-14,
-// 1.1e-13; s = 3: 7.2e-14, 1.1e-13 / 8.6e-14, 1.3e-13) nor for speed (64 nodes of 10 modes at
-// s = 3: 294 us / 1240 us), but because fixed-M iterations at third order end where rounding takes
+// with two of them 1e-5 apart, from both ends / from one: s = 2: 7.2e-14, 1.5e-13 / 8.4e-14,
+// 1.1e-13; s = 3: 9.1e-14, 1.0e-13 / 8.6e-14, 1.3e-13) nor for speed (64 nodes of 10 modes at
+// s = 3: 301 us / 1240 us), but because fixed-M iterations at third order end where rounding takes
 // them, and the order that the space-time refinement study shows at s = p = 3 depends on it.
 int taps_ts_ctas(const taps_problem* P, int hb, int M) {
   if (hb > 5 || M > 64 || P->ts_most < 1) return 0;
